@@ -68,28 +68,21 @@ typedef enum lrstv_status {
                                         2^-21); storage, the Jacobi and the thresholds stay
                                         FP32, the sigma-vs-threshold decisions FP64.  Not with
                                         LRSTV_FLAG_SIMT_GEMM (ERR_ARG). */
-#define LRSTV_FLAG_JACOBI_PER_SLICE 512u /* run each Fourier slice's Jacobi sweeps in one CTA
-                                        (its column panels in sequence) instead of the
-                                        task-graph schedule, in which every SM takes panel-pair
-                                        tasks of any slice (slices up to 256 rows; the same
-                                        t-SVT to rounding, the pairs visited in another
-                                        order).  Batches always run their slices this way, so
-                                        a batch's cube equals a plan made with this flag. */
+#define LRSTV_FLAG_JACOBI_PER_SLICE 512u /* accepted; without effect since the t-SVT's blocked
+                                        Jacobi, whose schedule never changes a result (it
+                                        chose one CTA per Fourier slice, which was the
+                                        batches' order of column pairs) */
 #define LRSTV_FLAG_SIMT_DFT 256u     /* the mode-3 (spectral) DFTs on the FP32 SIMT kernels (direct
                                         sums with twiddle tables) instead of the tensor-core
                                         pipeline (3xTF32, or 3xBF16 with LRSTV_FLAG_BF16X3);
                                         LRSTV_FLAG_SIMT_GEMM puts them there too */
-#define LRSTV_FLAG_JACOBI_PANEL16 1024u /* the Jacobi's column panels 16 wide, each CTA 8 warps
-                                        and two CTAs to an SM, instead of 32 wide with 16-warp
-                                        CTAs (slices up to 256 rows; the same t-SVT to
-                                        rounding, the pairs visited in another order).
-                                        Batches run 32-column panels whatever the flag. */
-#define LRSTV_FLAG_JACOBI_FIXED_ORDER 4096u /* the Jacobi pairs a slice's columns in their
-                                        stored order in every sweep, instead of ordering them
-                                        by squared norm, largest first, at the start of each
-                                        sweep (de Rijk's ordering: fewer sweeps; the same t-SVT
-                                        to rounding).  Slices of up to 256 rows, either
-                                        schedule; a batch follows its first cube's flag. */
+#define LRSTV_FLAG_JACOBI_PANEL16 1024u /* accepted; without effect: the blocked Jacobi's column
+                                        panels are 16 wide */
+#define LRSTV_FLAG_JACOBI_FIXED_ORDER 4096u /* the Jacobi takes a slice's columns in their stored
+                                        order instead of ordering them by squared norm,
+                                        largest first, at its start (de Rijk's ordering: fewer
+                                        sweeps; the same t-SVT to rounding).  A batch follows
+                                        its first cube's flag. */
 #define LRSTV_FLAG_UNROLL_RECOMPUTE 2048u /* unrolled iteration only: the forward pass keeps one
                                         slot of SVD factors instead of one per iteration, and
                                         the backward pass recomputes iteration k's factors
@@ -350,7 +343,7 @@ int lrstv_denoise(const float *Y, int n1, int n2, int n3, const lrstv_params *pa
  * The batch owns one plan per cube (lrstv_batch_plan lends it for stats and
  * state export; do not destroy it or change its parameters), one allocation
  * per group and one small allocation for the work list.  Slices taller than
- * 256 rows (max(n1, n2)) take a separate Jacobi launch per group.  The
+ * 256 rows (max(n1, n2)) take a separate Jacobi launch per cube.  The
  * persistent launch is recorded in cube 0's profile (lrstv_profile_*), a
  * group's other launches in the profile of its first cube.  A cube whose plan
  * has the Tucker L-update (lrstv_plan_set_tucker) takes its own launches for

@@ -48,13 +48,6 @@ int check_shape(int n1, int n2, int n3) {
 namespace {
 
 constexpr int kResRing = 4096;     // per-iteration residual history
-// SMs a plan's task-graph Jacobi leaves to the side stream, which runs the
-// next iteration's L-update and Z-solve while the E-step's Jacobi runs.  The
-// Jacobi's time follows the SMs it has (200 x 200 x 80: 5.05 ms on 152 SMs,
-// 5.52 on 136), while the side stream's work, once the Jacobi's CTAs have
-// left, takes a fraction of a millisecond on the whole GPU: 16 spare SMs gave
-// 155.4 iterations/s against 163.9 with none, so none are kept.
-constexpr int kJacobiSpareSMs = 0;
 
 int check_params(const lrstv_params *p) {
   if (!p) return LRSTV_ERR_ARG;
@@ -176,7 +169,7 @@ cudaError_t tsvt_pre(const Dims &d, int nb, const float *x, const float *y, floa
 // norms, which then set the threshold-aware tolerance tensor by tensor.
 cudaError_t tsvt_jac(const Dims &d, int nb, float t, float2 *specA, float2 *V, int *sweeps,
                      cudaStream_t st, Prof *prof, float *ms2 = nullptr, int *sched = nullptr,
-                     int pw = 32, int *order = nullptr, int sort = 1) {
+                     int sort = 1) {
   if (ms2) {
     cudaError_t e = launch_group_ms2(d, nb * d.h, specA, d.h, ms2, st);
     if (e != cudaSuccess) return e;
@@ -186,9 +179,6 @@ cudaError_t tsvt_jac(const Dims &d, int nb, float t, float2 *specA, float2 *V, i
   o.ms2 = ms2;
   o.group = d.h;
   o.sched = sched;
-  o.spare_sms = sched ? kJacobiSpareSMs : 0;
-  o.pw = pw;
-  o.order = order;
   o.sort = sort;
   Span sp(prof, LRSTV_K_JACOBI, st);
   return launch_jacobi(d, nb * d.h, specA, V, t, kMaxSweeps, sweeps, prof ? prof->d_work : nullptr,
@@ -218,11 +208,10 @@ cudaError_t tsvt_core(const Dims &d, int nb, const float *x, const float *y, flo
                       float *out, int mode, float *G4, const float *F, float mu, int gamma4,
                       const float2 *tw3, float2 *specA, float2 *specB, float2 *V, int *sweeps,
                       cudaStream_t st, Prof *prof = nullptr, GemmSel gs = kSimt,
-                      float *ms2 = nullptr, int *sched = nullptr, int pw = 32,
-                      int *order = nullptr, int sort = 1) {
+                      float *ms2 = nullptr, int *sched = nullptr, int sort = 1) {
   cudaError_t e = tsvt_pre(d, nb, x, y, ycoef, tw3, specA, st, prof, gs);
   if (e != cudaSuccess) return e;
-  if ((e = tsvt_jac(d, nb, t, specA, V, sweeps, st, prof, ms2, sched, pw, order, sort)) !=
+  if ((e = tsvt_jac(d, nb, t, specA, V, sweeps, st, prof, ms2, sched, sort)) !=
       cudaSuccess)
     return e;
   return tsvt_post(d, nb, out, mode, G4, F, mu, gamma4, tw3, specA, specB, V, st, prof, gs);
@@ -260,9 +249,8 @@ struct lrstv_plan {
   Tables tb;
   unsigned *res;  // kResRing x 2 residual maxima (float bits)
   int *sweeps;    // 3h
-  int *order;     // 3h: the one-CTA-per-slice Jacobi's slice order
   int *gcand, *gconv;  // 3h each: the tensor-core Gram check's candidates and flags
-  int *jsched;    // task-graph Jacobi scratch (jacobi_task_ints(3h))
+  int *jsched;    // scratch of the Jacobi's task schedule
   int *gemm_err;  // tensor-core GEMM wait timeouts
   // graph cache for lrstv_plan_run
   cudaGraphExec_t gexec;
@@ -295,15 +283,7 @@ struct lrstv_plan {
 
 namespace {
 
-// The task-graph Jacobi's scratch, or null for one CTA per slice.
-int *plan_sched(const lrstv_plan *pl) {
-  return (pl->prm.flags & LRSTV_FLAG_JACOBI_PER_SLICE) ? nullptr : pl->jsched;
-}
-
-// The packed Jacobi's panel width for a plan's flags.
-int plan_pw(const lrstv_plan *pl) { return (pl->prm.flags & LRSTV_FLAG_JACOBI_PANEL16) ? 16 : 32; }
-
-// Whether the task-graph Jacobi orders each sweep's columns by norm.
+// Whether the Jacobi orders a slice's columns by norm.
 int plan_sort(const lrstv_plan *pl) {
   return (pl->prm.flags & LRSTV_FLAG_JACOBI_FIXED_ORDER) ? 0 : 1;
 }
@@ -408,10 +388,7 @@ cudaError_t tsvt_warm(lrstv_plan *pl, float ycoef, float t, float mu, int gamma4
     o.t_svt = t;
     o.ms2 = pl->ms2;
     o.group = d.h;
-    o.sched = plan_sched(pl);
-    o.spare_sms = kJacobiSpareSMs;
-    o.pw = plan_pw(pl);
-    o.order = pl->order;
+    o.sched = pl->jsched;
     o.sort = plan_sort(pl);
     Span sp(&pl->prof, LRSTV_K_JACOBI, st);
     e = launch_jacobi(d, ns, Wm, pl->V, -1.0f, kMaxSweeps, pl->sweeps,
@@ -487,10 +464,10 @@ size_t group_layout(lrstv_plan *const *pls, int m, void *base) {
   for (int i = 0; i < m; ++i) pls[i]->tb = tb;
   take_each(c, pls, m, 2 * (size_t)kResRing, &lrstv_plan::res);
   take_each(c, pls, m, 3 * h, &lrstv_plan::sweeps);
-  take_each(c, pls, m, 3 * h, &lrstv_plan::order);
   take_each(c, pls, m, 3 * h, &lrstv_plan::gcand);
   take_each(c, pls, m, 3 * h, &lrstv_plan::gconv);
-  take_each(c, pls, m, (size_t)jacobi_task_ints(3 * d.h), &lrstv_plan::jsched);
+  take_each(c, pls, m, jacobi_task_ints(3 * d.h, d.nc, 3 * h * jacobi_op_bytes(d.nr, d.nc)),
+            &lrstv_plan::jsched);
   take_each(c, pls, m, 1, &lrstv_plan::gemm_err);
   unsigned long long *work = c.take<unsigned long long>(2 * (size_t)m);
   for (int i = 0; i < m; ++i) pls[i]->prof.d_work = work ? work + 2 * (size_t)i : nullptr;
@@ -941,7 +918,7 @@ int lrstv_step_e(lrstv_plan *pl, void *stream) {
   CK(tsvt_core(pl->d, 3, pl->F, pl->G4, (float)(1.0 / mu), (float)(pl->prm.alpha / mu), pl->E, 1,
                pl->G4, pl->F, (float)mu, gamma4, pl->tb.tw3, pl->specA, pl->specB, pl->V,
                pl->sweeps, (cudaStream_t)stream, &pl->prof, plan_gemm(pl), pl->ms2,
-               plan_sched(pl), plan_pw(pl), pl->order, plan_sort(pl)));
+               pl->jsched, plan_sort(pl)));
   return LRSTV_OK;
 }
 
@@ -1115,6 +1092,8 @@ int lrstv_plan_autotune(lrstv_plan *pl, const float *Y, int iters, unsigned allo
     if ((sub & ~allowed) != 0) continue;
     // SIMT_GEMM already puts the DFTs on the SIMT kernels
     if ((sub & LRSTV_FLAG_SIMT_GEMM) && (sub & LRSTV_FLAG_SIMT_DFT)) continue;
+    // these two change nothing: timing them would only repeat a candidate
+    if (sub & (LRSTV_FLAG_JACOBI_PER_SLICE | LRSTV_FLAG_JACOBI_PANEL16)) continue;
     lrstv_params trial = pl->prm;
     trial.flags = base | sub;
     if (check_params(&trial) == LRSTV_OK && nc < 64) cands[nc++] = base | sub;
@@ -1211,10 +1190,8 @@ struct lrstv_batch {
   void *arena;           // the slice work list and its counter
   SliceTask *d_tasks;
   int ntasks;
-  int *d_counter;
-  int grid;
-  size_t smem;
-  int max_nr;  // the tallest slice in the persistent work list
+  int *d_sched;          // the task queue's scratch
+  int max_nr, max_nc;    // the largest slice sides in the work list
   cudaStream_t cap_stream;
   cudaGraphExec_t gexec;
   const float **gY;
@@ -1329,27 +1306,29 @@ int batch_e_step(lrstv_batch *b, cudaStream_t st) {
     }
   }
   if (b->ntasks > 0) {
-    CK(cudaMemsetAsync(b->d_counter, 0, sizeof(int), st));
     Prof *prof = &b->plans[0]->prof;
     Span sp(prof, LRSTV_K_JACOBI, st);
-    CK(launch_jacobi_batch(b->d_tasks, b->ntasks, b->d_counter, mu, kMaxSweeps,
-                           prof->on ? prof->d_work : nullptr, b->grid, b->smem, st, warm,
-                           wflag ? 1 : 0, b->max_nr, plan_sort(b->plans[0])));
+    CK(launch_jacobi_list(b->d_tasks, b->ntasks, b->max_nr, b->max_nc, mu, kMaxSweeps,
+                          prof->on ? prof->d_work : nullptr, st, warm, wflag ? 1 : 0,
+                          plan_sort(b->plans[0]), b->d_sched));
   }
   for (int k = 0; k < b->ngroups; ++k) {
     const BatchGroup &g = b->groups[k];
     if (!g.big) continue;
-    lrstv_plan *p = g.pls[0];
-    Span sp(&p->prof, LRSTV_K_JACOBI, st);
-    JacOpt o;
-    o.warm = warm;
-    o.t_svt = (float)(p->prm.alpha / mu);
-    o.ms2 = p->ms2;
-    o.group = p->d.h;
-    o.order = p->order;
-    o.sort = plan_sort(p);
-    CK(launch_jacobi(p->d, 3 * p->d.h * g.m, p->specA, p->V, wflag ? -1.0f : o.t_svt,
-                     kMaxSweeps, p->sweeps, p->prof.on ? p->prof.d_work : nullptr, st, o));
+    for (int i = 0; i < g.m; ++i) {
+      lrstv_plan *p = g.pls[i];
+      Span sp(&p->prof, LRSTV_K_JACOBI, st);
+      JacOpt o;
+      o.conv = wflag && plan_gemm(p).tc ? p->gconv : nullptr;
+      o.warm = warm;
+      o.t_svt = (float)(p->prm.alpha / mu);
+      o.ms2 = p->ms2;
+      o.group = p->d.h;
+      o.sched = p->jsched;
+      o.sort = plan_sort(p);
+      CK(launch_jacobi(p->d, 3 * p->d.h, p->specA, p->V, wflag ? -1.0f : o.t_svt, kMaxSweeps,
+                       p->sweeps, p->prof.on ? p->prof.d_work : nullptr, st, o));
+    }
   }
   for (int k = 0; k < b->ngroups; ++k) {
     const BatchGroup &g = b->groups[k];
@@ -1503,12 +1482,14 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
     batch_free(b);
     return rc;
   }
-  int ntasks = 0, maxnr = 1;
+  int ntasks = 0, maxnr = 1, maxnc = 1;
+  size_t op = 0;
   for (int i = 0; i < ncubes; ++i) {
     const Dims &d = b->plans[i]->d;
     if (d.nr <= kBatchMaxNr) {
       ntasks += 3 * d.h;
       if (d.nr > maxnr) maxnr = d.nr;
+      if (d.nc > maxnc) maxnc = d.nc;
     }
   }
   b->ntasks = ntasks;
@@ -1534,33 +1515,32 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
         // the Gram check runs with the warm start on the tensor-core engine
         h[k].conv = ((pl->prm.flags & LRSTV_FLAG_WARM_START) && plan_gemm(pl).tc)
                         ? pl->gconv + s : nullptr;
+        h[k].op = op;
+        op += jacobi_op_bytes(d.nr, d.nc);
         ++k;
       }
     }
     qsort(h, (size_t)ntasks, sizeof(SliceTask), task_cmp);
     const size_t tbytes = align_up(sizeof(SliceTask) * (size_t)ntasks);
-    int dev = 0, sms = 1;
-    if (cudaMalloc(&b->arena, tbytes + kAlign) != cudaSuccess) {
+    if (cudaMalloc(&b->arena, tbytes + sizeof(int) * jacobi_task_ints(ntasks, maxnc, op)) !=
+        cudaSuccess) {
       cudaGetLastError();
       delete[] h;
       batch_free(b);
       return LRSTV_ERR_ALLOC;
     }
     b->d_tasks = (SliceTask *)b->arena;
-    b->d_counter = (int *)((char *)b->arena + tbytes);
+    b->d_sched = (int *)((char *)b->arena + tbytes);
     const bool ok = cudaMemcpy(b->d_tasks, h, sizeof(SliceTask) * (size_t)ntasks,
-                               cudaMemcpyHostToDevice) == cudaSuccess &&
-                    cudaGetDevice(&dev) == cudaSuccess &&
-                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+                               cudaMemcpyHostToDevice) == cudaSuccess;
     delete[] h;
     if (!ok) {
       cudaGetLastError();
       batch_free(b);
       return LRSTV_ERR_CUDA;
     }
-    b->grid = ntasks < sms ? ntasks : sms;  // one 512-thread CTA fills an SM's registers
-    b->smem = jacobi_batch_smem(maxnr);
     b->max_nr = maxnr;
+    b->max_nc = maxnc;
   }
   if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
@@ -1693,14 +1673,18 @@ static size_t zsolve_ws(const Dims &d, Tables *tb, float2 **A, float2 **B, void 
   return c.off;
 }
 
+// *sched: the task queue's scratch, after the rest (*least: the bytes without
+// it; a smaller workspace runs one CTA per slice)
 static size_t tsvt_ws(const Dims &d, float2 **tw, float2 **A, float2 **B, float2 **V, int **sw,
-                      void *base) {
+                      int **sched, size_t *least, void *base) {
   Carver c(base);
   *A = c.take<float2>((size_t)d.h * d.P);
   *B = c.take<float2>((size_t)d.h * d.P);
   *V = c.take<float2>((size_t)d.h * d.nc * d.nc);
   *tw = c.take<float2>(d.n3);
   *sw = c.take<int>(d.h);
+  *least = c.off;
+  *sched = c.take<int>(jacobi_task_ints(d.h, d.nc, d.h * jacobi_op_bytes(d.nr, d.nc)));
   return c.off;
 }
 
@@ -1719,8 +1703,9 @@ int lrstv_tsvt_workspace_size(int n1, int n2, int n3, size_t *bytes) {
   int rc = check_shape(n1, n2, n3);
   if (rc) return rc;
   float2 *tw, *a, *b, *v;
-  int *sw;
-  *bytes = tsvt_ws(make_dims(n1, n2, n3), &tw, &a, &b, &v, &sw, nullptr);
+  int *sw, *sched;
+  size_t least;
+  *bytes = tsvt_ws(make_dims(n1, n2, n3), &tw, &a, &b, &v, &sw, &sched, &least, nullptr);
   return LRSTV_OK;
 }
 
@@ -1749,13 +1734,15 @@ int lrstv_tsvt(const float *Ain, int n1, int n2, int n3, float t, float *out, vo
   if (!isfinite(t) || t < 0.0f || ((size_t)workspace % kAlign)) return LRSTV_ERR_ARG;
   const Dims d = make_dims(n1, n2, n3);
   float2 *tw, *A, *B, *V;
-  int *sw;
-  if (tsvt_ws(d, &tw, &A, &B, &V, &sw, nullptr) > workspace_bytes) return LRSTV_ERR_ARG;
-  tsvt_ws(d, &tw, &A, &B, &V, &sw, workspace);
+  int *sw, *sched;
+  size_t least;
+  const size_t full = tsvt_ws(d, &tw, &A, &B, &V, &sw, &sched, &least, workspace);
+  if (least > workspace_bytes) return LRSTV_ERR_ARG;
+  if (full > workspace_bytes) sched = nullptr;
   cudaStream_t st = (cudaStream_t)stream;
   CK(launch_tw3(d.n3, tw, st));
   CK(tsvt_core(d, 1, Ain, nullptr, 0.0f, t, out, 0, nullptr, nullptr, 0.0f, 0, tw, A, B, V, sw,
-               st));
+               st, nullptr, kSimt, nullptr, sched));
   if (sweeps_host) {
     int *h = new (std::nothrow) int[d.h];
     if (!h) return LRSTV_ERR_ALLOC;

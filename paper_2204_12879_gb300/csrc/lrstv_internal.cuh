@@ -161,27 +161,16 @@ struct JacOpt {
   const float *ms2 = nullptr;
   int group = 1;
   float negl_rel = -1.0f;
-  // scratch of jacobi_task_ints(nslices) ints: with it, slices of up to 256
-  // rows run on the task-graph schedule (all SMs share every slice's panel
-  // pairs); without it, one CTA per slice
+  // scratch of jacobi_task_ints(nslices, nc, nslices jacobi_op_bytes(nr, nc))
+  // ints: with it, every SM takes tasks of any slice from a queue; without it,
+  // one CTA runs a slice
   int *sched = nullptr;
-  // SMs the task-graph grid leaves free for concurrent work (another stream's
-  // kernels cannot share an SM with a worker CTA, which takes its shared memory)
-  int spare_sms = 0;
-  // panel width of the packed kernels (slices of up to 256 rows): 32 columns
-  // with 16-warp CTAs, or 16 with 8-warp CTAs, two to an SM
-  int pw = 32;
-  // scratch of nslices ints: with it, the one-CTA-per-slice kernel starts the
-  // slices in the order of their sweeps in the previous run (the sweeps array
-  // as passed in), most first, so that long slices do not end a wave alone
-  int *order = nullptr;
   // nslices flags of launch_gram_check (may be null): a slice whose flag is
   // set ends after one sweep without running it (that sweep would rotate
   // no pair)
   const int *conv = nullptr;
-  // packed kernels (slices of up to 256 rows, either schedule): each sweep
-  // pairs the slice's columns in the order of their squared norms, largest
-  // first (0: in the stored order)
+  // each sweep pairs the slice's columns in the order of their squared norms,
+  // largest first (0: in the stored order)
   int sort = 1;
 };
 // The Jacobi's base tolerance for slices of nr rows: a pair is rotated when
@@ -199,11 +188,20 @@ float jacobi_tol0(int nr);
 cudaError_t launch_gram_check(const Dims &d, int nslices, const float2 *W, float2 *G,
                               const int *sweeps, int *cand, int *conv, float t_svt,
                               const float *ms2, int group, int *gemm_err, cudaStream_t st);
-// ints of task-graph scratch for nslices working matrices
-size_t jacobi_task_ints(int nslices);
+// Scratch of the blocked kernel's task schedule: bytes of one slice's operands,
+// and ints for nslices working matrices of up to nc columns whose operands
+// take op_total bytes (256-byte aligned).
+size_t jacobi_op_bytes(int nr, int nc);
+size_t jacobi_task_ints(int nslices, int nc, size_t op_total);
+// The blocked kernel (jacobi_blk.cu), or, when negl_rel is given (the Tucker
+// eigen-solves, whose null-space columns the blocked kernel's FP16 halves
+// would not resolve), the per-slice FP32 kernels (svt.cu).
 cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, float t,
                           int max_sweeps, int *sweeps, unsigned long long *work,
                           cudaStream_t st, const JacOpt &opt = JacOpt());
+cudaError_t launch_jacobi_blk(const Dims &d, int nslices, float2 *W, float2 *V, float t,
+                              int max_sweeps, int *sweeps, unsigned long long *work,
+                              cudaStream_t st, const JacOpt &opt);
 // ms2[g] = max over slices s of group g (s / group == g) of ||W_s||_F^2 / nc.
 cudaError_t launch_group_ms2(const Dims &d, int nslices, const float2 *W, int group, float *ms2,
                              cudaStream_t st);
@@ -228,16 +226,18 @@ struct SliceTask {
   int nr, nc;
   const float *ms2;  // the slice's group value of launch_group_ms2 (may be null)
   const int *conv;   // the slice's launch_gram_check flag (may be null)
+  size_t op;         // the slice's operands: their offset in the scratch's operand part
 };
-// Largest slice height the persistent batch kernel takes.
-constexpr int kBatchMaxNr = 256;  // the packed kernel's tallest slice
-size_t jacobi_batch_smem(int max_nr);
-// Persistent work-list Jacobi over `ntasks` slices; *counter must be 0.  warm:
-// as launch_jacobi; keep: V left unscaled (threshold taken as negative).
-// max_nr: the tallest slice (up to 256 rows).  sort: as JacOpt::sort.
-cudaError_t launch_jacobi_batch(const SliceTask *tasks, int ntasks, int *counter, double mu,
-                                int max_sweeps, unsigned long long *work, int grid, size_t smem,
-                                cudaStream_t st, int warm, int keep, int max_nr, int sort);
+// Largest slice height of a batch's common launch (taller slices would leave
+// one CTA to an SM for all of them).
+constexpr int kBatchMaxNr = 256;
+// The blocked Jacobi over a list of slices of any shapes up to max_nr x max_nc.
+// warm: as launch_jacobi; keep: V left unscaled (threshold taken as negative);
+// sort: as JacOpt::sort; sched: jacobi_task_ints(nslices, max_nc, the slices'
+// jacobi_op_bytes together) ints.
+cudaError_t launch_jacobi_list(const SliceTask *list, int nslices, int max_nr, int max_nc,
+                               double mu, int max_sweeps, unsigned long long *work,
+                               cudaStream_t st, int warm, int keep, int sort, int *sched);
 
 // ------------------------------------------------------------------- api.cu
 constexpr size_t kAlign = 256;

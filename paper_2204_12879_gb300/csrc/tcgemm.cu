@@ -41,6 +41,7 @@
 #include <stdint.h>
 
 #include "lrstv_internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace lrstv {
 
@@ -52,12 +53,6 @@ constexpr int TN = 64;        // complex columns of C per CTA
 // and, by warpgroup, columns 0..31 or 32..63 of each Re / Im tile
 constexpr int kThreads = 256;
 constexpr uint32_t kLBO = 128;  // bytes
-// tries of a bounded barrier wait: one mbarrier.try_wait that finds the
-// phase incomplete suspends the thread for about 3.8 us on GB300 (measured
-// by the wait probe below), so the bound is about a second, against the
-// microseconds one chunk's MMAs take
-constexpr long long kWaitLimit = 250000;
-
 // Per precision: element bytes, elements per 16-byte core-matrix row, the
 // 8-row group stride, tile sizes and the instruction descriptor's operand
 // format (kind::tf32: TF32 = 2; kind::f16: BF16 = 1).
@@ -76,17 +71,9 @@ struct Prec {
   static constexpr size_t kTileB = (size_t)TN * kKR * kBytes;     // bytes, one split, re or im
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
 template <int PREC>
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-  uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
-  d |= (uint64_t)((kLBO >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((Prec<PREC>::kSBO >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of tcgen05; no swizzle, base offset 0
-  return d;
+  return tc_desc(addr, kLBO, Prec<PREC>::kSBO);
 }
 
 // byte offset of element (row r, real k kk) in a K-major no-swizzle tile
@@ -139,20 +126,6 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
-                                          long long tries = kWaitLimit) {
-  uint32_t done = 0;
-  for (long long it = 0; it < tries && !done; ++it) {
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-  }
-  return done != 0;
 }
 
 // KIND 0: the complex GEMM C = A op(B) of CGemm (OPB 0: B, 1: B^H), or, with

@@ -390,7 +390,7 @@ struct lrstv_unroll {
   double *sig;
   float2 *Hs;          // 3 B h nc^2 complex: thresholded V, then H / K'
   int *sweeps;         // K x 3 B h
-  int *jsched;         // task-graph Jacobi scratch (jacobi_task_ints(3 B h))
+  int *jsched;         // scratch of the Jacobi's task schedule
   float *ms2;          // 3 B: per gradient tensor, largest mean-square column norm
   int *gemm_err;
   Tables tb;
@@ -447,7 +447,7 @@ size_t unroll_layout(lrstv_unroll *u, void *base) {
   u->sig = c.take<double>((size_t)u->nw * ns * d.nc);
   u->Hs = c.take<float2>(ns * d.nc * d.nc);
   u->sweeps = c.take<int>((size_t)u->K * ns);
-  u->jsched = c.take<int>(jacobi_task_ints((int)ns));
+  u->jsched = c.take<int>(jacobi_task_ints((int)ns, d.nc, ns * jacobi_op_bytes(d.nr, d.nc)));
   u->ms2 = c.take<float>((size_t)3 * u->B);
   u->gemm_err = c.take<int>(1);
   carve_tables(c, d, u->tb);
@@ -514,8 +514,7 @@ int e_factor(lrstv_unroll *u, int k, const float *F, const float *G4, double mu,
   o.t_svt = t;
   o.ms2 = u->ms2;
   o.group = d.h;
-  o.sched = (u->flags & LRSTV_FLAG_JACOBI_PER_SLICE) ? nullptr : u->jsched;
-  o.pw = (u->flags & LRSTV_FLAG_JACOBI_PANEL16) ? 16 : 32;
+  o.sched = u->jsched;
   o.sort = (u->flags & LRSTV_FLAG_JACOBI_FIXED_ORDER) ? 0 : 1;
   UCK(launch_jacobi(d, (int)ns, Wk, Vk, -1.0f, kMaxSweeps, u->sweeps + (size_t)k * ns, nullptr,
                     st, o));
