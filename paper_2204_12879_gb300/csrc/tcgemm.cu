@@ -288,13 +288,8 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
         const int gm = m0 + r, gk = k0 + kc;
         if (KIND == 2) {  // raw; conjugated (transposed slices) when stored
           ra[i] = (gm < gM && gk < gK) ? specb[wpos(gm) + f.P * gk] : make_float2(0.f, 0.f);
-        } else if (OPB == 2) {  // A^H(m, k) = conj A(k, m)
-          float2 v = make_float2(0.f, 0.f);
-          if (gm < g.M && gk < g.K) {
-            v = A[gk + (size_t)g.lda * gm];
-            v.y = -v.y;
-          }
-          ra[i] = v;
+        } else if (OPB == 2) {  // A^H(m, k) = conj A(k, m): conjugated when stored
+          ra[i] = (gm < g.M && gk < g.K) ? A[gk + (size_t)g.lda * gm] : make_float2(0.f, 0.f);
         } else {
           ra[i] = (gm < g.M && gk < g.K) ? A[gm + (size_t)g.lda * gk] : make_float2(0.f, 0.f);
         }
@@ -305,12 +300,11 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
           int n, kc;
           b_pos(i, n, kc);
           const int gn = n0 + n, gk = k0 + kc;
-          float2 v = make_float2(0.f, 0.f);
-          if (gn < g.N && gk < g.K) {
-            v = OPB != 1 ? B[gk + (size_t)g.ldb * gn] : B[gn + (size_t)g.ldb * gk];
-            if (OPB == 1) v.y = -v.y;
-          }
-          rb[i] = v;
+          // raw (OPB 1: conjugated when stored): combining a value where it is
+          // loaded makes the thread wait for it there
+          rb[i] = (gn < g.N && gk < g.K)
+                      ? (OPB != 1 ? B[gk + (size_t)g.ldb * gn] : B[gn + (size_t)g.ldb * gk])
+                      : make_float2(0.f, 0.f);
         }
       }
     }
@@ -323,6 +317,7 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
     b_pos(i, n, kc);
     if (KIND == 0) {
       v = rb[i];
+      if (OPB == 1) v.y = -v.y;
     } else if (KIND == 1) {
       v = twid(n0 + n, k0 + kc);
       w = twid(n0 + n, k0 + TK + kc);
@@ -350,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
         const float2 w = ry[KIND == 1 ? i : 0];
         v = make_float2(v.x - f.ycoef * w.x, v.y - f.ycoef * w.y);
       }
-      if (KIND == 2 && f.trans) v.y = -v.y;
+      if ((KIND == 2 && f.trans) || (KIND == 0 && OPB == 2)) v.y = -v.y;
       return v;
     };
     if (PREC == 0) {
