@@ -99,6 +99,33 @@ __device__ __forceinline__ bool wsync_and(bool v) {
 }
 // barriers of the whole CTA: workers and the ninth warp
 __device__ __forceinline__ void csync() { asm volatile("bar.sync 2, 288;" ::: "memory"); }
+// ... and of a rotation round's copy c, where one side arrives without waiting:
+// its state is published (the ninth warp waits), its rotations are formed (the
+// workers wait)
+__device__ __forceinline__ void state_arrive(int c) {
+  if (c)
+    asm volatile("bar.arrive 4, 288;" ::: "memory");
+  else
+    asm volatile("bar.arrive 3, 288;" ::: "memory");
+}
+__device__ __forceinline__ void state_sync(int c) {
+  if (c)
+    asm volatile("bar.sync 4, 288;" ::: "memory");
+  else
+    asm volatile("bar.sync 3, 288;" ::: "memory");
+}
+__device__ __forceinline__ void formed_arrive(int c) {
+  if (c)
+    asm volatile("bar.arrive 6, 288;" ::: "memory");
+  else
+    asm volatile("bar.arrive 5, 288;" ::: "memory");
+}
+__device__ __forceinline__ void formed_sync(int c) {
+  if (c)
+    asm volatile("bar.sync 6, 288;" ::: "memory");
+  else
+    asm volatile("bar.sync 5, 288;" ::: "memory");
+}
 
 __host__ __device__ inline int panels_of(int nc) { return (nc + kB - 1) / kB; }
 // with an empty panel that makes an odd number even
@@ -422,7 +449,7 @@ struct Smem {
   char *A, *S;
   uint32_t bar[2], bar_w, bar_v, bar_task, bar_done, bar_vdone;
   uint32_t tmem;     // 128 columns: the Gram, then two 64-column update tiles
-  float4 *par;       // 2 x 16: a round's rotations (m, sigma; 0 in .w: no pair rotates)
+  float4 *par;       // 2 x 16: a round's rotations (m, sigma)
   float2 *piv;       // 16: the first round's G(p, q)
   float *diag;       // 32: G's diagonal at first
   unsigned *rounds;  // the rounds that rotate a pair
@@ -434,7 +461,18 @@ struct Rot2 {
 
 // whether a pair is rotated: beyond the tolerance, no column negligible
 __device__ __forceinline__ bool rotates(float al, float be, float g2, const float4 &lim) {
-  return al > lim.y && be > lim.y && g2 > lim.x * (al * be) && g2 > lim.z * fmaxf(al, be);
+  return (al > lim.y) & (be > lim.y) & (g2 > lim.x * (al * be)) & (g2 > lim.z * fmaxf(al, be));
+}
+
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // Rotation of the Hermitian [[al, g], [conj g, be]], g2 = |g|^2, by the smaller
@@ -445,14 +483,14 @@ __device__ __forceinline__ bool rotates(float al, float be, float g2, const floa
 // from the sigma that is applied.
 __device__ __forceinline__ Rot2 make_rot2(float al, float be, float2 g, float g2, float &shift) {
   const float d = 0.5f * (be - al);
-  const float ih = rsqrtf(fmaf(d, d, g2));
+  const float ih = rsqrt_ftz(fmaf(d, d, g2));
   const float c2 = fmaf(0.5f * fabsf(d), ih, 0.5f);
-  const float ic = rsqrtf(c2);
+  const float ic = rsqrt_ftz(c2);
   const float f = copysignf(0.5f * ih * ic, d);  // sin / |g|
   Rot2 r;
   r.sr = f * g.x;
   r.si = -f * g.y;
-  r.m = __fdividef(-(f * f) * g2, fmaf(c2, ic, 1.0f));
+  r.m = -(f * f) * g2 * rcp_ftz(fmaf(c2, ic, 1.0f));
   shift = f * g2 * ic;
   return r;
 }
@@ -519,7 +557,11 @@ struct Waits {
 
 // The rotations' shared state (sm.S and sm.par): a round's rotations, its
 // state of G, and the blocks that the next round's rotations come from, in two
-// copies, so that one barrier a round suffices.
+// copies.  A worker that has rotated G publishes state r + 1 without waiting,
+// rotates Q, and then waits for round r + 1's rotations (and so for the other
+// workers' states); the ninth warp forms them from state r meanwhile.  With one
+// barrier of all a round, both chains had to end before either went on: 600
+// cycles a round; with mbarriers in place of the hardware's named ones, 900.
 // Across the panels, round r pairs a_k with b_(k + r); only the rounds in which
 // some pair is beyond the tolerance at first are run (a pair that other
 // rotations push beyond it waits for the next sweep; about a third of the
@@ -632,18 +674,19 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
 
   float4 qa = make_float4(k == 2 * i ? 1.f : 0.f, k == 2 * i + 1 ? 1.f : 0.f, 0.f, 0.f);
   float4 qb = make_float4(16 + k == 2 * i ? 1.f : 0.f, 16 + k == 2 * i + 1 ? 1.f : 0.f, 0.f, 0.f);
-  auto apply = [&](const float4 &u, const float4 &v) {  // its columns' rotations, its rows'
-    const Rot2 rk = {u.x, u.y, u.z}, ri = {v.x, v.y, v.z};
+  auto apply_g = [&](const Rot2 &rk, const Rot2 &ri) {  // its columns' rotations, its rows'
     rot_cols(aa, ab, rk);
     rot_cols(ba, bb, rk);
+    rot_rows(aa, ba, ri);
+    rot_rows(ab, bb, ri);
+  };
+  auto apply_q = [&](const Rot2 &rk) {
     float2 x = make_float2(qa.x, qa.z), y = make_float2(qb.x, qb.z);
     rot_cols(x, y, rk);
     float2 z = make_float2(qa.y, qa.w), w = make_float2(qb.y, qb.w);
     rot_cols(z, w, rk);
     qa = make_float4(x.x, z.x, x.y, z.y);
     qb = make_float4(y.x, w.x, y.y, w.y);
-    rot_rows(aa, ba, ri);
-    rot_rows(ab, bb, ri);
   };
   auto shfl4 = [](float4 v, int src) {
     return make_float4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
@@ -651,20 +694,26 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
   };
   if (own) {
     const int w = 32 * i + k;
+    state_arrive(0);
     for (int r = 0; r < 31; ++r) {
-      csync();
+      formed_sync(r & 1);
       const float2 *G = A->G[r & 1];
       float2 *N = A->G[(r + 1) & 1];
+      const float4 u = sm.par[16 * (r & 1) + k], v = sm.par[16 * (r & 1) + i];
+      const Rot2 rk = {u.x, u.y, u.z}, ri = {v.x, v.y, v.z};
       aa = G[ga + ca];
       ab = G[ga + cb];
       ba = G[gb + ca];
       bb = G[gb + cb];
-      const float4 u = sm.par[16 * (r & 1) + k], v = sm.par[16 * (r & 1) + i];
-      if (u.w != 0.f) apply(u, v);  // else no pair of the round rotates
-      N[w] = aa;
-      N[w + 16] = ab;
-      N[w + 512] = ba;
-      N[w + 528] = bb;
+      apply_g(rk, ri);
+      if (r < 30) {
+        N[w] = aa;
+        N[w + 16] = ab;
+        N[w + 512] = ba;
+        N[w + 528] = bb;
+        state_arrive((r + 1) & 1);
+      }
+      apply_q(rk);
       const float4 t = shfl4(k == 0 ? qb : qa, (lane & 16) | ((k + 15) & 15));
       const float4 z = shfl4(qb, (lane & 16) | ((k + 1) & 15));
       qb = k == 15 ? qa : z;
@@ -673,38 +722,45 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
   } else {
     // to the first round, whose pairs the ninth warp takes from piv
     unsigned left = rounds & (rounds - 1);
-    int r = __ffs(rounds) - 1, d = r, kd = (k + d) & 15;
+    int r = __ffs(rounds) - 1, d = r, d2 = after(left, r);
     if (k == ((i + d) & 15)) sm.piv[i] = ab;
-    auto move = [&](int n, int d2) {  // copy n: d rounds on; d2: the move after this
+    // G into copy n for a state d rounds on, d2 the move after that (block (i, i + d2)
+    // of that state: its ab is still d columns on here), then the columns
+    auto move = [&](int n, bool pa, bool pb) {
       X->BA[n][tid] = ba;
       X->BB[n][tid] = bb;
-      const int from = (lane & 16) | kd;
+      if (pa) X->AX[n][i] = aa;
+      if (pb) X->AB[n][i] = ab;
+      state_arrive(n);
+    };
+    auto columns = [&](int from) {
       ab.x = __shfl_sync(0xffffffffu, ab.x, from);
       ab.y = __shfl_sync(0xffffffffu, ab.y, from);
       qb = shfl4(qb, from);
-      if (k == ((i + d2) & 15)) {
-        X->AX[n][i] = aa;
-        X->AB[n][i] = ab;
-      }
     };
-    int d2 = after(left, r);
-    move(0, d2);
-    csync();  // piv is there
+    move(0, k == ((i + d2) & 15), k == ((i + d + d2) & 15));
+    columns((lane & 16) | ((k + d) & 15));
     auto step = [&](int c) -> bool {  // a round on copy c; true after the last
+      // what does not wait for the round comes before it
       const int row = (tid + 16 * d) & 0xff;
-      const float2 *pa = X->BA[c] + row, *pb = X->BB[c] + ((row & 0xf0) | kd);
-      csync();
-      ba = *pa;
-      bb = *pb;
-      apply(sm.par[16 * c + k], sm.par[16 * c + i]);
-      if (!left) return true;
+      const float2 *pa = X->BA[c] + row, *pb = X->BB[c] + ((row & 0xf0) | ((k + d) & 15));
+      const bool last = !left;
       d = d2;
       r += d;
-      kd = (k + d) & 15;
       left &= left - 1;
       d2 = after(left, r);
-      move(c ^ 1, d2);
-      return false;
+      const int from = (lane & 16) | ((k + d) & 15);
+      const bool ea = k == ((i + d2) & 15), eb = k == ((i + d + d2) & 15);
+      formed_sync(c);
+      const float4 u = sm.par[16 * c + k], v = sm.par[16 * c + i];
+      const Rot2 rk = {u.x, u.y, u.z}, ri = {v.x, v.y, v.z};
+      ba = *pa;
+      bb = *pb;
+      apply_g(rk, ri);
+      if (!last) move(c ^ 1, ea, eb);
+      apply_q(rk);
+      if (!last) columns(from);
+      return last;
     };
     while (!step(0) && !step(1)) {
     }
@@ -769,7 +825,7 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
   const Whole *A = (const Whole *)sm.S;
   int r = own ? 0 : __ffs(left) - 1, d = r;
   left &= left - 1;
-  if (!own) csync();
+  state_sync(0);
   float al = sm.diag[k], be = sm.diag[16 + ((k + r) & 15)];
   float2 g = sm.piv[k];
   Rot2 t;
@@ -779,14 +835,9 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
     const bool go = rotates(al, be, g2, lim);
     t = make_rot2(al, be, g, g2, shift);
     if (!go) t.m = t.sr = t.si = shift = 0.f;
-    if (own) {
-      const unsigned any = __ballot_sync(0xffffffffu, go) & 0xffffu;
-      if (lane < 16) sm.par[16 * c + lane] = make_float4(t.m, t.sr, t.si, any ? 1.f : 0.f);
-      n_rot += __popc(any);
-    } else {
-      if (lane < 16) sm.par[16 * c + lane] = make_float4(t.m, t.sr, t.si, 1.f);
-      n_rot += __popc(__ballot_sync(0xffffffffu, go) & 0xffffu);
-    }
+    if (lane < 16) sm.par[16 * c + lane] = make_float4(t.m, t.sr, t.si, 0.f);
+    formed_arrive(c);
+    n_rot += __popc(__ballot_sync(0xffffffffu, go) & 0xffffu);
   };
   form(0);
   if (own) {
@@ -804,7 +855,7 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
       const float ay = __shfl_sync(0xffffffffu, a1, ky), by = __shfl_sync(0xffffffffu, b1, ky);
       al = xb ? bx : ax;
       be = yb ? by : ay;
-      csync();
+      if (r > 0) state_sync(r & 1);
       if (r == 30) break;
       const float2 *G = A->G[r & 1];
       const float2 tt = G[rt + ct], tu = G[rt + cu], ut = G[ru + ct], uu = G[ru + cu];
@@ -818,6 +869,7 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
     }
   } else {
     int d2 = after(left, r);
+    bool first = true;  // the first state has been waited for
     for (int c = 0;; c ^= 1) {
       // what does not wait for the workers comes before the barrier
       const int k2 = (k + d2) & 15, row = ((k + d) & 15) * 16;
@@ -826,7 +878,8 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
                   si1 = __shfl_sync(0xffffffffu, t.si, k2);
       al -= shift;
       be = __shfl_sync(0xffffffffu, be + shift, k2);
-      csync();
+      if (!first) state_sync(c);
+      first = false;
       if (!left) break;
       const float2 aa = X->AX[c][k], ab = X->AB[c][k], ba = *pa, bb = *pb;
       const float2 va = rot_one(ab, aa, m1, sr1, -si1), vb = rot_one(bb, ba, m1, sr1, -si1);
@@ -1474,10 +1527,11 @@ cudaError_t blk_launch(Run a, cudaStream_t st) {
     return e;
   const int fit = (int)((size_t)sm_smem / (smem + at.sharedSizeBytes + 1024));
   const int per_sm = fit < 1 ? 1 : (fit > 3 ? 3 : fit);
-  // workers: the resident CTAs, and no more than the tasks a round offers
+  // workers: the resident CTAs, and no more than twice the tasks a round offers
+  // (a CTA that updates V leaves the next round's W to another)
   const int width = players_of(panels_of(a.cols)) / 2;
   long long grid = (long long)per_sm * nsm;
-  if (grid > (long long)a.nslices * width) grid = (long long)a.nslices * width;
+  if (grid > 2ll * a.nslices * width) grid = 2ll * a.nslices * width;
   // slices in flight: their operands within about 96 MB of the 129 MB L2, and
   // enough of them to give every worker two tasks
   const long long bytes = (long long)op_bytes(a.nr, a.nc);
