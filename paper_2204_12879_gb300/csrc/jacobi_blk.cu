@@ -34,8 +34,8 @@
 // column takes in a cold 200-column run); with m it does not.
 //
 // Layout.  During a run W and V live in scratch, as the MMA operands that the
-// tasks read: a panel is 8 groups (Re hi of its columns 0-7 and 8-15, Im hi,
-// then the low halves alike), a group holds 16 bytes (8 columns) of every row,
+// tasks read: a panel is 8 groups (Re hi of its columns 0-7 and 8-15, Re lo,
+// then Im alike), a group holds 16 bytes (8 columns) of every row,
 // rows contiguous.  A task's panels then arrive by two bulk copies with no
 // instruction spent on them, and serve the update as the K-major A operand
 // and the Gram as both MN-major operands.
@@ -49,7 +49,7 @@
 //
 // What bounds it: the latency of a task's chain (16 rotation rounds of two
 // barriers each, two loads, three MMA waits); 72 registers and one region of
-// shared memory for W and then V let three CTAs share an SM at 200 rows.
+// shared memory for W and then V let three CTAs share an SM up to 256 rows.
 #include <cuda_fp16.h>
 #include <float.h>
 
@@ -65,7 +65,15 @@ constexpr int kW = 256;             // worker threads
 constexpr int kT = kW + 32;         // and the ninth warp: rotations, scheduling
 constexpr int kMaxTasks = 16;       // tasks of a round: 512 columns in 32 panels
 constexpr int kMaxRounds = 32;
-constexpr size_t kScratch = 16384;  // Gram dump, then G and Q, then Q as an operand
+// The scratch holds the Gram's dump, then G, then Q as an operand.  In 10 KB the
+// dump takes two passes and Q's lo has no -Im Q of its own; in 16 KB (kWide)
+// neither holds, which is 1.5% faster in whole runs (sixteen cubes of 64 to 200
+// columns, 12 iterations: 464 ms against 471) and is taken unless it costs an SM
+// a CTA: with 10 KB three CTAs of 256 rows fit instead of two (256 x 256 x 191,
+// 16 iterations with BF16X3: 250.9 -> 223.5 ms).
+template <bool kWide>
+constexpr size_t kScratch = kWide ? 16384 : 10240;
+constexpr uint32_t kLoQ = 6144;  // Q's lo in the operand
 constexpr float kScaleV = 8192.0f, kScaleQ = 16384.0f;
 // A pair is left alone when the component of the smaller column along the
 // larger is below kAbsTol ||W||_F: 1e-3 of an FP32 rounding of ||W||_F, and
@@ -74,9 +82,12 @@ constexpr float kAbsTol = 1e-3f * 0.5f * FLT_EPSILON;
 constexpr unsigned long long kTaskWaitNs = 2000000000ull;  // a wait for work gives up after 2 s
 constexpr long long kWorkerWait = 2000000;  // tries of a worker's wait for its scheduler (about 8 s)
 
-// f16 operands, F32 accumulator, M = 128: the update (N = 64, K-major
-// operands) and the Gram (N = 128, MN-major operands: transpose bits 15, 16)
+// f16 operands, F32 accumulator, M = 128: the update (K-major operands; N = 64 or
+// 32, bit 13: A negated) and the Gram (N = 128, MN-major operands: transpose bits
+// 15, 16)
 constexpr uint32_t kIdescUpd = (1u << 4) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kIdescUpdIm = (1u << 4) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kIdescUpdRe = kIdescUpdIm | (1u << 13);
 constexpr uint32_t kIdescGram =
     (1u << 4) | (1u << 15) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
@@ -125,6 +136,12 @@ __device__ __forceinline__ void formed_sync(int c) {
     asm volatile("bar.sync 6, 288;" ::: "memory");
   else
     asm volatile("bar.sync 5, 288;" ::: "memory");
+}
+// ... and where one state of G has one copy: it has been read by all (the ninth
+// warp does not wait)
+__device__ __forceinline__ void state_read() { asm volatile("bar.sync 7, 288;" ::: "memory"); }
+__device__ __forceinline__ void state_read_arrive() {
+  asm volatile("bar.arrive 7, 288;" ::: "memory");
 }
 
 __host__ __device__ inline int panels_of(int nc) { return (nc + kB - 1) / kB; }
@@ -409,14 +426,14 @@ __device__ __forceinline__ void put_row(char *dst, int rows, int row, int g, con
     re[j] = x[j].x * scale;
     im[j] = x[j].y * scale;
   }
-  const size_t step = (size_t)rows * 32;  // Re hi, Im hi, Re lo, Im lo: two groups each
+  const size_t step = (size_t)rows * 32;  // Re hi, Re lo, Im hi, Im lo: two groups each
   char *d = dst + ((size_t)g * rows + row) * 16;
   uint4 hi, lo;
   split8(re, hi, lo);
   *(uint4 *)d = hi;
-  *(uint4 *)(d + 2 * step) = lo;
+  *(uint4 *)(d + step) = lo;
   split8(im, hi, lo);
-  *(uint4 *)(d + step) = hi;
+  *(uint4 *)(d + 2 * step) = hi;
   *(uint4 *)(d + 3 * step) = lo;
 }
 
@@ -444,7 +461,7 @@ __device__ __forceinline__ void pack_panels(char *dst, const float2 *M, int n, i
 }
 
 // Shared memory of one CTA: the pair's columns of W, then of V, as operands
-// (`A`: panel a's 8 groups, then panel b's), and 16 KB of scratch (`S`).
+// (`A`: panel a's 8 groups, then panel b's), and the scratch (`S`).
 struct Smem {
   char *A, *S;
   uint32_t bar[2], bar_w, bar_v, bar_task, bar_done, bar_vdone;
@@ -519,20 +536,34 @@ __device__ __forceinline__ void issue_gram(uint32_t d, uint32_t a, int rows, uin
   tc_commit(bar);
 }
 
-// The MMAs of one 128-row tile of an update: D (128 x 64) = tile (Q - I), the
-// small split products first (one thread).
+// The MMAs of one 128-row tile of an update: D (128 x 64: Re, then Im, of both
+// panels' columns) = tile (Q - I), the small split products first (one thread).
+// The columns' real parts meet [Re Q, Im Q], their imaginary parts [-Im Q, Re Q]:
+// two windows of Q's hi, which holds -Im Q, Re Q and Im Q; where the lo has no
+// -Im Q, two MMAs with N = 32, one with A negated, take its place.
+template <bool kWide>
 __device__ __forceinline__ void issue_update(uint32_t d, uint32_t a, int rows, uint32_t q,
                                              uint32_t bar) {
-  const uint64_t x = tc_desc(a, (uint32_t)rows * 16, 128), y = tc_desc(q, 1024, 128);
+  const uint64_t x = tc_desc(a, (uint32_t)rows * 16, 128), y = tc_desc(q, 1536, 128),
+                 z = tc_desc(q + kLoQ, kWide ? 1536 : 1024, 128);
+  const uint32_t lo = (uint32_t)(2 * rows);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {  // Re a, Im a, Re b, Im b
-    const uint64_t xk = x + (uint32_t)(((k & 1) * 2 + (k >> 1) * 8) * rows);
-    tc_mma_f16(d, xk, y + 512 + 128 * k, kIdescUpd, k > 0 ? 1u : 0u);
-    tc_mma_f16(d, xk + (uint32_t)(4 * rows), y + 128 * k, kIdescUpd, 1u);
+    const uint64_t xk = x + (uint32_t)(4 * k * rows);
+    const uint32_t at = 192 * (k >> 1) + ((k & 1) ? 0 : 32);
+    const uint64_t yk = y + at, zk = z + (kWide ? at : 128 * (k >> 1));
+    if (!kWide && (k & 1)) {
+      tc_mma_f16(d, xk, zk + 32, kIdescUpdRe, 1u);
+      tc_mma_f16(d + 32, xk, zk, kIdescUpdIm, 1u);
+    } else {
+      tc_mma_f16(d, xk, zk, kIdescUpd, k > 0 ? 1u : 0u);
+    }
+    tc_mma_f16(d, xk + lo, yk, kIdescUpd, 1u);
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    tc_mma_f16(d, x + (uint32_t)(((k & 1) * 2 + (k >> 1) * 8) * rows), y + 128 * k, kIdescUpd, 1u);
+    tc_mma_f16(d, x + (uint32_t)(4 * k * rows),
+               y + 192 * (k >> 1) + ((k & 1) ? 0 : 32), kIdescUpd, 1u);
   tc_commit(bar);
 }
 
@@ -571,7 +602,8 @@ struct Waits {
 // round after's pairs are published in AX (aa) and AB (ab).
 // All 32 columns (the first round's tasks): a tournament of 31 rounds in which
 // pair k is (a_k, b_k) and after a round a_0 stays, a_1 := b_0, a_k := a_(k-1),
-// b_k := b_(k+1), b_15 := a_15; G moves through shared memory.
+// b_k := b_(k+1), b_15 := a_15; G moves through shared memory, in one copy that
+// is rewritten when all workers and the ninth warp have read it.
 __device__ __forceinline__ int from_a(int j) { return j == 0 ? 0 : (j == 1 ? 16 : j - 1); }
 __device__ __forceinline__ int from_b(int j) { return j == 15 ? 15 : 17 + j; }
 // the round after round r in the mask of those left (0: none)
@@ -580,14 +612,15 @@ struct Cross {
   float2 BA[2][256], BB[2][256], AX[2][16], AB[2][16];
 };
 struct Whole {
-  float2 G[2][1024];
+  float2 G[1024];
 };
-static_assert(sizeof(Cross) <= kScratch && sizeof(Whole) <= kScratch, "the scratch holds them");
+static_assert(sizeof(Cross) <= kScratch<false> && sizeof(Whole) <= kScratch<false>, "the scratch holds them");
 
 // Steps 1 and 2 of a task by the worker warps, W's operands being in sm.A
 // (`rows` rows; ok: warp 0 saw them arrive): G, the rotations, and Q - I as an operand in
 // sm.S.  Returns 1 (rotated), 0 (no pair needed it) or -1 (a wait ran out).
 // The ninth warp runs form_rotations beside it.
+template <bool kWide>
 __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim, Waits &wt,
                            bool ok) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -602,41 +635,70 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
   }
   // Thread (i, k) holds the 2 x 2 block of G's rows a_i, b_i and columns a_k, b_k
   // (a_j, b_j: column j of panel a, of panel b) and Q's rows 2i, 2i + 1 there.
-  // D's rows and columns: panel, hi/lo, Re/Im, column (1, 1, 1, 4 bits).  Half
-  // h: the columns that are Re (0) or Im (1), hi + lo, to S[column][row]; a row
-  // is XOR-ed with its column's parity, so that the two i of a warp read
-  // different banks.  G(p, q) = conj(w_p) . w_q is read as conj(G(q, p)): the
-  // lanes' q are D's rows.
+  // D's rows and columns: panel, Re/Im, hi/lo, column (1, 1, 1, 4 bits).  A lane
+  // adds hi and lo of its row's columns, then the lanes l and l + 16 (a row's hi
+  // and lo) exchange halves: l keeps the sums of the columns' Re (h = 0), l + 16
+  // of their Im.  The rows that are Re, then those that are Im, go to
+  // S[h][column][row], the row XOR-ed so that the two i of a warp read different
+  // banks.
+  // G(p, q) = conj(w_p) . w_q is read as conj(G(q, p)): the lanes' q are D's rows.
   const int i = tid >> 4, k = tid & 15;
   float *S = (float *)sm.S;
   float2 aa, ab, ba, bb;
+  {
+    const uint32_t at = sm.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64 * (warp >> 2);
+    float x[16];
+    {
+      uint32_t v[16], w[16];
+      tc_ld16(at, v);
+      tc_ld16(at + 16, w);
+      tc_wait_ld();
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const uint32_t at =
-        sm.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64 * (warp >> 2) + 16 * h;
-    uint32_t v[16], w[16];
-    tc_ld16(at, v);
-    tc_ld16(at + 32, w);
-    tc_wait_ld();
-    float *d = S + (16 * (warp >> 2)) * 128;
-    const int m = 32 * (warp & 3) + lane;
+      for (int j = 0; j < 16; ++j) x[j] = __uint_as_float(v[j]) + __uint_as_float(w[j]);
+      tc_ld16(at + 32, v);
+      tc_ld16(at + 48, w);
+      tc_wait_ld();
+      const bool up = lane > 15;
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
-      d[j * 128 + (m ^ (16 * (j & 1)))] = __uint_as_float(v[j]) + __uint_as_float(w[j]);
-    wsync();
-    auto part = [&](int n, int q, float2 &g) {
-      const float *x = S + n * 128 + 64 * q, *re = x + (k ^ (16 * (i & 1))),
-                  *im = x + ((16 + k) ^ (16 * (i & 1)));
-      const float r = re[0] + re[32], u = im[0] + im[32];  // (Re q, Im q) . (Re p or Im p)
-      if (h == 0)
-        g = make_float2(r, u);
-      else
-        g = make_float2(g.x + u, g.y - r);
+      for (int j = 0; j < 16; ++j) {
+        const float y = __uint_as_float(v[j]) + __uint_as_float(w[j]);
+        x[j] = (up ? y : x[j]) + __shfl_xor_sync(0xffffffffu, up ? x[j] : y, 16);
+      }
+    }
+    float *d = S + (kWide ? 2048 * (warp & 1) : 0) + 1024 * (lane >> 4) + 512 * (warp >> 2) + k;
+    const int f = 16 * (((warp >> 1) ^ (lane >> 4)) & 1);
+    auto store = [&]() {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) d[32 * j + (f ^ (16 * (j & 1)))] = x[j];
     };
-    part(i, 0, aa);
-    part(i, 1, ab);
-    part(16 + i, 0, ba);
-    part(16 + i, 1, bb);
+    if (kWide || !(warp & 1)) store();
+    wsync();
+    auto part = [&](int n, int q, float &re, float &im) {  // q . Re p, q . Im p
+      const float *y = S + 32 * n + k;
+      const int e = 16 * ((q ^ i) & 1);
+      re = y[e];
+      im = y[1024 + 16 - e];
+    };
+    part(i, 0, aa.x, aa.y);
+    part(i, 1, ab.x, ab.y);
+    part(16 + i, 0, ba.x, ba.y);
+    part(16 + i, 1, bb.x, bb.y);
+    if (kWide) {
+      S += 2048;
+    } else {
+      wsync();
+      if (warp & 1) store();
+      wsync();
+    }
+    auto second = [&](int n, int q, float2 &g) {
+      float re, im;
+      part(n, q, re, im);
+      g = make_float2(g.x + im, re - g.y);
+    };
+    second(i, 0, aa);
+    second(i, 1, ab);
+    second(16 + i, 0, ba);
+    second(16 + i, 1, bb);
     wsync();
   }
   // the diagonal, and the rounds in which a pair needs a rotation
@@ -649,10 +711,10 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
     if (own) sm.piv[k] = ab;
   }
   if (own) {
-    A->G[0][ga + ca] = aa;
-    A->G[0][ga + cb] = ab;
-    A->G[0][gb + ca] = ba;
-    A->G[0][gb + cb] = bb;
+    A->G[ga + ca] = aa;
+    A->G[ga + cb] = ab;
+    A->G[gb + ca] = ba;
+    A->G[gb + cb] = bb;
   }
   wsync();
   {
@@ -697,8 +759,7 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
     state_arrive(0);
     for (int r = 0; r < 31; ++r) {
       formed_sync(r & 1);
-      const float2 *G = A->G[r & 1];
-      float2 *N = A->G[(r + 1) & 1];
+      float2 *G = A->G;
       const float4 u = sm.par[16 * (r & 1) + k], v = sm.par[16 * (r & 1) + i];
       const Rot2 rk = {u.x, u.y, u.z}, ri = {v.x, v.y, v.z};
       aa = G[ga + ca];
@@ -707,10 +768,11 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
       bb = G[gb + cb];
       apply_g(rk, ri);
       if (r < 30) {
-        N[w] = aa;
-        N[w + 16] = ab;
-        N[w + 512] = ba;
-        N[w + 528] = bb;
+        state_read();
+        G[w] = aa;
+        G[w + 16] = ab;
+        G[w + 512] = ba;
+        G[w + 528] = bb;
         state_arrive((r + 1) & 1);
       }
       apply_q(rk);
@@ -766,9 +828,9 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
     }
     qb = shfl4(qb, (lane & 16) | ((k + 16 - r) & 15));  // home
   }
-  // Q - I as the K-major operand (64 x 64): output n = panel, Re/Im, column;
-  // input = panel, Re/Im, column: [[Re, Im], [-Im, Re]], hi and lo.  This
-  // thread: inputs 2i and 2i + 1 (one 4-byte word), outputs a_k and b_k.
+  // Q - I as the K-major operand: output n = -Im (see issue_update), Re, Im times panel
+  // and column; input = panel, column.  This thread: inputs 2i and 2i + 1 (one
+  // 4-byte word), outputs a_k and b_k.
   wsync();
   {
     const int d = k - 2 * i;  // 0, 1: the diagonal is in a_k; 16, 17 below: in b_k
@@ -776,24 +838,22 @@ __device__ int gram_rotate(const Smem &sm, int rows, bool own, const float4 &lim
     qa.y -= d == 1 ? 1.f : 0.f;
     qb.x -= d + 16 == 0 ? 1.f : 0.f;
     qb.y -= d + 16 == 1 ? 1.f : 0.f;
-    // input 2i: panel i >> 3, column 2 (i & 7): its Re in k-group 4 (i >> 3) +
-    // ((i & 7) >> 2), its Im two groups on
-    char *re = sm.S + (4 * (i >> 3) + ((i & 7) >> 2)) * 1024 + (i & 3) * 4;
-    auto put = [&](char *at, float x, float y) {
+    // inputs 2i, 2i + 1: k-group i >> 2
+    char *hi = sm.S + (i >> 2) * 1536 + 512 + (i & 3) * 4 + k * 16;
+    char *lo = kWide ? hi + kLoQ : sm.S + kLoQ + (i >> 2) * 1024 + (i & 3) * 4 + k * 16;
+    auto put = [&](int at, float x, float y, bool im) {
       const __half2 h = __floats2half2_rn(x * kScaleQ, y * kScaleQ);
       const float2 f = __half22float2(h);
-      *(__half2 *)at = h;
-      *(__half2 *)(at + 8192) = __floats2half2_rn(fmaf(x, kScaleQ, -f.x), fmaf(y, kScaleQ, -f.y));
+      const __half2 l = __floats2half2_rn(fmaf(x, kScaleQ, -f.x), fmaf(y, kScaleQ, -f.y));
+      *(__half2 *)(hi + at) = h;
+      *(__half2 *)(lo + at) = l;
+      if (im) *(__half2 *)(hi + at - 1024) = __hneg2(h);
+      if (im && kWide) *(__half2 *)(lo + at - 1024) = __hneg2(l);
     };
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const float4 x = p ? qb : qa;
-      char *at = re + (32 * p + k) * 16;
-      put(at, x.x, x.y);               // Re -> Re
-      put(at + 256, x.z, x.w);         // Re -> Im
-      put(at + 2048, -x.z, -x.w);      // Im -> Re
-      put(at + 2048 + 256, x.x, x.y);  // Im -> Im
-    }
+    put(0, qa.x, qa.y, false);
+    put(256, qb.x, qb.y, false);
+    put(512, qa.z, qa.w, true);
+    put(768, qb.z, qb.w, true);
   }
   tc_fence_smem();
   tc_fence_before();
@@ -857,8 +917,9 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
       be = yb ? by : ay;
       if (r > 0) state_sync(r & 1);
       if (r == 30) break;
-      const float2 *G = A->G[r & 1];
+      const float2 *G = A->G;
       const float2 tt = G[rt + ct], tu = G[rt + cu], ut = G[ru + ct], uu = G[ru + cu];
+      state_read_arrive();
       // column y: a' = a + m a - sigma b, b' = b + m b + conj(sigma) a
       const float cr = yb ? sry : -sry;
       const float2 vt = rot_one(yb ? tu : tt, yb ? tt : tu, my, cr, -siy);
@@ -896,8 +957,8 @@ __device__ unsigned form_rotations(const Smem &sm, bool own, const float4 &lim) 
 
 // Step 3 for the operands in sm.A (`rows` rows): every 128-row tile's product
 // with Q - I is added to it and handed, eight columns at a time, to
-// put(panel, group 0..1 of Re (0, 1) or Im (2, 3), row, values).
-template <class Put>
+// put(panel, Re (0) or Im (1), its group 0..1, row, values).
+template <bool kWide, class Put>
 __device__ bool update(const Smem &sm, int rows, Waits &wt, Put put) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pan = warp >> 2;
   const int tiles = (rows + 127) / 128;
@@ -907,29 +968,29 @@ __device__ bool update(const Smem &sm, int rows, Waits &wt, Put put) {
     if (tid == 0) {
       tc_fence_after();
       for (int i = 0; i < n; ++i)
-        issue_update(sm.tmem + 64 * i, smem_u32(sm.A) + (t0 + i) * 2048, rows, smem_u32(sm.S),
-                     sm.bar[i]);
+        issue_update<kWide>(sm.tmem + 64 * i, smem_u32(sm.A) + (t0 + i) * 2048, rows,
+                            smem_u32(sm.S), sm.bar[i]);
     }
     wt.out |= (1u << n) - 1u;
     for (int i = 0; i < n; ++i) {
       if (!wt.mma(sm, i, true)) return false;
       const int row = 128 * (t0 + i) + 32 * (warp & 3) + lane;
-      const uint32_t at = sm.tmem + 64 * i + ((uint32_t)(32 * (warp & 3)) << 16) + 32 * pan;
+      const uint32_t at = sm.tmem + 64 * i + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * pan;
       const char *src = sm.A + 8 * pan * grp + row * 16;
 #pragma unroll
       for (int part = 0; part < 2; ++part) {
         uint32_t acc[16];
-        tc_ld16(at + 16 * part, acc);
+        tc_ld16(at + 32 * part, acc);
         tc_wait_ld();
         if (row < rows) {
 #pragma unroll
           for (int g = 0; g < 2; ++g) {
-            const char *p = src + (2 * part + g) * grp;
+            const char *p = src + (4 * part + g) * grp;
             float x[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) x[j] = __uint_as_float(acc[8 * g + j]) * (1.0f / kScaleQ);
-            join8(*(const uint4 *)p, *(const uint4 *)(p + 4 * grp), x);
-            put(pan, 2 * part + g, row, x);
+            join8(*(const uint4 *)p, *(const uint4 *)(p + 2 * grp), x);
+            put(pan, part, g, row, x);
           }
         }
       }
@@ -1064,8 +1125,8 @@ __global__ void __launch_bounds__(256) k_blk_close(Run a) {
         const char *b = src + ((size_t)g * rows + r) * 16;
         const size_t st = (size_t)rows * 32;
         float re[8] = {}, im[8] = {};
-        join8(*(const uint4 *)b, *(const uint4 *)(b + 2 * st), re);
-        join8(*(const uint4 *)(b + st), *(const uint4 *)(b + 3 * st), im);
+        join8(*(const uint4 *)b, *(const uint4 *)(b + st), re);
+        join8(*(const uint4 *)(b + 2 * st), *(const uint4 *)(b + 3 * st), im);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int c = s_col[8 * g + j];
@@ -1143,6 +1204,7 @@ struct TaskInfo {
 // The task schedule: a persistent grid whose CTAs take tasks of any slice until
 // every slice has ended (or a wait runs out; slices still open then stay
 // reported as capped).
+template <bool kWide>
 __global__ void __launch_bounds__(kT, 3) k_jacobi_tasks(Run a) {
   extern __shared__ __align__(128) char smem[];
   __shared__ __align__(8) uint64_t s_bar[7];
@@ -1170,19 +1232,19 @@ __global__ void __launch_bounds__(kT, 3) k_jacobi_tasks(Run a) {
       if (!wsync_and(warp != 0 || mbar_wait(sm.bar_task, k & 1u, kWorkerWait))) break;
       const TaskInfo ti = s_info;
       if (ti.rw < 0) break;
-      int rot = gram_rotate(sm, ti.rw, ti.own, ti.lim, wt,
+      int rot = gram_rotate<kWide>(sm, ti.rw, ti.own, ti.lim, wt,
                             warp != 0 || mbar_wait(sm.bar_w, k & 1u));
       if (rot > 0) {
         auto put_to = [&](char *pa, char *pb, int rows) {
-          return [=](int pan, int g, int row, const float (&x)[8]) {
+          return [=](int pan, int part, int g, int row, const float (&x)[8]) {
             uint4 hi, lo;
             split8(x, hi, lo);
-            char *d = (pan ? pb : pa) + (g * rows + row) * 16;
+            char *d = (pan ? pb : pa) + ((4 * part + g) * rows + row) * 16;
             __stcg((uint4 *)d, hi);
-            __stcg((uint4 *)(d + rows * 64), lo);
+            __stcg((uint4 *)(d + rows * 32), lo);
           };
         };
-        if (!update(sm, ti.rw, wt, put_to(ti.wa, ti.wb, ti.rw))) rot = -1;
+        if (!update<kWide>(sm, ti.rw, wt, put_to(ti.wa, ti.wb, ti.rw))) rot = -1;
         fence_async();  // the columns' next readers are bulk copies
         // every thread has read W's operands: the ninth warp lets V's take their place
         if (tid == 0) s_rot = rot;
@@ -1191,7 +1253,7 @@ __global__ void __launch_bounds__(kT, 3) k_jacobi_tasks(Run a) {
         if (rot > 0) {
           const bool here = wsync_and(warp != 0 || mbar_wait(sm.bar_v, v_ph, kWorkerWait));
           v_ph ^= 1u;
-          if (!here || !update(sm, ti.rv, wt, put_to(ti.va, ti.vb, ti.rv))) rot = -1;
+          if (!here || !update<kWide>(sm, ti.rv, wt, put_to(ti.va, ti.vb, ti.rv))) rot = -1;
           fence_async();
         }
       } else {
@@ -1408,7 +1470,7 @@ __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
   sm.diag = s_diag;
   sm.rounds = &s_rounds;
   sm.piv = s_piv;
-  int *perm = (int *)(sm.S + kScratch);
+  int *perm = (int *)(sm.S + kScratch<false>);
   cta_begin(sm, s_bar, &s_tmem);
   Waits wt;
   unsigned n_pairs = 0, n_rot = 0;
@@ -1436,7 +1498,7 @@ __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
     };
     // both parts of a value meet here: Re is written first, then Im
     auto put_to = [&](float2 *M, int n, float inv) {
-      return [=](int pan, int g, int row, const float (&v)[8]) {
+      return [=](int pan, int part, int g, int row, const float (&v)[8]) {
         uint4 hi, lo;
         float f[8] = {};
         split8(v, hi, lo);
@@ -1444,8 +1506,8 @@ __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
         if (row >= n) return;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int c = s_cols[kB * pan + 8 * (g & 1) + j];
-          if (c >= 0) ((float *)(M + (size_t)n * c + row))[g >> 1] = f[j] * inv;
+          const int c = s_cols[kB * pan + 8 * g + j];
+          if (c >= 0) ((float *)(M + (size_t)n * c + row))[part] = f[j] * inv;
         }
       };
     };
@@ -1465,12 +1527,12 @@ __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
           n_pairs += wa * wb + (r == 0 ? (wa * (wa - 1) + wb * (wb - 1)) / 2 : 0);
           if (worker) {
             load(x.W, x.nr, rw, 1.0f / lim.w);
-            int rot = gram_rotate(sm, rw, r == 0, lim, wt, true);
+            int rot = gram_rotate<false>(sm, rw, r == 0, lim, wt, true);
             if (rot > 0) {
-              bool ok = update(sm, rw, wt, put_to(x.W, x.nr, lim.w));
+              bool ok = update<false>(sm, rw, wt, put_to(x.W, x.nr, lim.w));
               if (ok) {
                 load(x.V, x.nc, rv, kScaleV);
-                ok = update(sm, rv, wt, put_to(x.V, x.nc, 1.0f / kScaleV));
+                ok = update<false>(sm, rv, wt, put_to(x.V, x.nc, 1.0f / kScaleV));
               }
               if (!ok) rot = -1;
             }
@@ -1501,32 +1563,43 @@ __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
 }
 
 cudaError_t blk_launch(Run a, cudaStream_t st) {
-  int dev = 0, nsm = 0;
-  const bool tasks = a.sched != nullptr;
-  const size_t smem = (size_t)a.rows * 256 + kScratch + (tasks ? 0 : sizeof(int) * (size_t)a.cols);
-  const void *f = tasks ? (const void *)k_jacobi_tasks : (const void *)k_jacobi_slices;
-  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  if (!tasks) {
+  int dev = 0, nsm = 0, sm_smem = 0, cta_smem = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) !=
+          cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&cta_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
+          cudaSuccess)
+    return e;
+  const size_t ops = (size_t)a.rows * 256;
+  // resident CTAs of an SM, by shared memory (1 KB a CTA is the system's),
+  // registers (three by the launch bounds) and TMEM (128 of 512 columns a CTA);
+  // cudaOccupancyMaxActiveBlocksPerMultiprocessor says 1 of this kernel.  The
+  // dynamic limit is the same for every size: threads may launch at once.
+  auto prepare = [&](const void *f, size_t smem, int &per_sm) -> cudaError_t {
+    cudaFuncAttributes at;
+    cudaError_t r = cudaFuncGetAttributes(&at, f);
+    if (r != cudaSuccess) return r;
+    const int fit = (int)((size_t)sm_smem / (smem + at.sharedSizeBytes + 1024));
+    per_sm = fit < 1 ? 1 : (fit > 3 ? 3 : fit);
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                cta_smem - (int)at.sharedSizeBytes);
+  };
+  int per_sm = 0, per_sm_wide = 0;
+  if (!a.sched) {
+    const size_t smem = ops + kScratch<false> + sizeof(int) * (size_t)a.cols;
+    if ((e = prepare((const void *)k_jacobi_slices, smem, per_sm)) != cudaSuccess) return e;
     k_jacobi_slices<<<a.nslices, kT, smem, st>>>(a);
     return cudaGetLastError();
   }
   a.cap = queue_cap(a.nslices);
   a.op = (char *)(a.sched + Sched::ints(a.nslices, a.cap, a.cols));
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+  if ((e = prepare((const void *)k_jacobi_tasks<false>, ops + kScratch<false>, per_sm)) !=
+          cudaSuccess ||
+      (e = prepare((const void *)k_jacobi_tasks<true>, ops + kScratch<true>, per_sm_wide)) !=
+          cudaSuccess)
     return e;
-  // resident CTAs of an SM, by shared memory (1 KB a CTA is the system's),
-  // registers (three by the launch bounds) and TMEM (128 of 512 columns a CTA);
-  // cudaOccupancyMaxActiveBlocksPerMultiprocessor says 1 of this kernel
-  int sm_smem = 0;
-  cudaFuncAttributes at;
-  if ((e = cudaFuncGetAttributes(&at, f)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) !=
-      cudaSuccess)
-    return e;
-  const int fit = (int)((size_t)sm_smem / (smem + at.sharedSizeBytes + 1024));
-  const int per_sm = fit < 1 ? 1 : (fit > 3 ? 3 : fit);
   // workers: the resident CTAs, and no more than twice the tasks a round offers
   // (a CTA that updates V leaves the next round's W to another)
   const int width = players_of(panels_of(a.cols)) / 2;
@@ -1543,7 +1616,10 @@ cudaError_t blk_launch(Run a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   k_blk_setup<<<a.nslices, 1024, 0, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_jacobi_tasks<<<(unsigned)grid, kT, smem, st>>>(a);
+  if (per_sm_wide == per_sm)
+    k_jacobi_tasks<true><<<(unsigned)grid, kT, ops + kScratch<true>, st>>>(a);
+  else
+    k_jacobi_tasks<false><<<(unsigned)grid, kT, ops + kScratch<false>, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_blk_close<<<dim3(a.nslices, panels_of(a.cols)), 256, 0, st>>>(a);
   return cudaGetLastError();
