@@ -90,6 +90,7 @@ struct CGemm {
   // tensor-core kernel only (may be null): batch entry b is computed only
   // where gate[b] != 0 (the other entries' C is left as it is)
   const int *gate;
+  int fold, slice_m;  // set by the tensor-core launch: slices of slice_m rows as one matrix
 };
 cudaError_t launch_cgemm(const CGemm &g, cudaStream_t st);
 
@@ -119,7 +120,6 @@ struct Dft3 {
 };
 cudaError_t launch_dft3_tc(int kind, const Dft3 &f, int nb, int *err, cudaStream_t st,
                            int prec = 0);
-size_t cgemm_tc_smem();
 // the tries of the GEMM's bounded barrier wait, and a one-warp check of that
 // wait and its timeout path (out: two device ints, zeroed by the caller)
 long long cgemm_tc_wait_limit();

@@ -25,15 +25,26 @@
 // MMA instructions of 3xTF32 (K = 16 per instruction instead of 8).
 //
 // Tile: 128 rows of C (M = 128 MMA), 64 complex columns (one N = 128 MMA over
-// the adjacent Re and Im B tiles into 128 TMEM columns, which reads the A tile
-// once for both parts), 8 (3xTF32) or 16 (3xBF16) complex K per chunk: two
-// K = 8 TF32 or two K = 16 BF16 MMA steps per product, a 32 KB stage either
-// way.  Operands are staged by the CTA's threads into shared memory in the
-// canonical K-major layout without swizzle: 8-row x 16-byte core matrices,
-// K-adjacent core matrices 128 B apart (LBO), 8-row groups one chunk row
-// (KR elements) apart (SBO).  Two stages and two TMEM tiles pipeline the
-// chunks: chunk k is loaded and staged while chunk k - 1's MMAs run, and
-// chunk k - 1's tile is drained while chunk k's MMAs run.
+// adjacent Re and Im B blocks into 128 TMEM columns, which reads the A tile
+// once for both parts), 8 (3xTF32) or 16 (3xBF16) complex K per chunk: the
+// chunk's real parts are one MMA's K, its imaginary parts the other's; 28 KB a
+// stage.  Operands are staged by the CTA's threads into shared memory in the
+// canonical K-major layout without swizzle: 8-row x 16-byte core matrices, the
+// two of an MMA's K 128 B apart (LBO), 8-row groups 256 B apart (SBO).  B is
+// held as the blocks -Im, Re, Im: [Re | Im] meets A's real parts, [-Im | Re] its
+// imaginary ones.
+//
+// What bounds it: the instructions that stage the operands; the tensor core's
+// part of a chunk is a third.  A thread therefore owns one row of A and a run of
+// consecutive k, a whole 16-byte row of a core matrix (B: half of one): its
+// bounds and addresses are worked out once, a chunk's loads walk along K, and a
+// run goes to shared memory in one store.  With an element's position worked
+// out at a time and 4-byte stores, 123 slices of 200 x 200 took 114 us instead
+// of 105 (3xTF32; 288 of 256 x 256 with 3xBF16 249 instead of 200), and the
+// forward DFT of three 200 x 200 x 80 cubes 71 instead of 41.
+// Two stages and two TMEM tiles pipeline the chunks: chunk k is loaded and
+// staged while chunk k - 1's MMAs run, and chunk k - 1's tile is drained while
+// chunk k's MMAs run.
 // One thread issues the MMAs and commits them to the stage's mbarrier; every
 // wait on a barrier is bounded and, if it runs out, the CTA records an error
 // flag, skips its epilogue and still frees its tensor memory.
@@ -52,37 +63,29 @@ constexpr int TN = 64;        // complex columns of C per CTA
 // eight warps: warp w reads TMEM lanes 32 (w mod 4) .. + 31 (rows of the tile)
 // and, by warpgroup, columns 0..31 or 32..63 of each Re / Im tile
 constexpr int kThreads = 256;
-constexpr uint32_t kLBO = 128;  // bytes
-// Per precision: element bytes, elements per 16-byte core-matrix row, the
-// 8-row group stride, tile sizes and the instruction descriptor's operand
+constexpr uint32_t kLBO = 128, kSBO = 256;  // bytes
+// Per precision: element bytes, the K of one MMA (two core matrices, 32 bytes of a
+// row), the elements of a core matrix's row and the instruction descriptor's operand
 // format (kind::tf32: TF32 = 2; kind::f16: BF16 = 1).
 template <int PREC>
 struct Prec {
   static constexpr int kBytes = PREC ? 2 : 4;
-  // complex K per chunk: 8 for 3xTF32 (16 real terms per TMEM tile), 16 for
-  // 3xBF16; either way a stage is 32 KB and two stages fit two CTAs per SM
-  static constexpr int kTK = PREC ? 16 : 8;
-  static constexpr int kKR = 2 * kTK;                             // real K per chunk
-  static constexpr int kPerCore = 16 / kBytes;                    // along K
-  static constexpr uint32_t kSBO = (kKR / kPerCore) * 128;        // bytes
-  static constexpr int kMmaK = PREC ? 16 : 8;                     // K per instruction
+  static constexpr int kTK = 32 / kBytes;   // complex K per chunk: 16 real terms per TMEM
+  static constexpr int kKR = 2 * kTK;       // tile with 3xTF32
+  static constexpr int kRun = 16 / kBytes;
   static constexpr uint32_t kFmt = PREC ? 1u : 2u;
-  static constexpr size_t kTileA = (size_t)TM * kKR * kBytes;     // bytes, one split
-  static constexpr size_t kTileB = (size_t)TN * kKR * kBytes;     // bytes, one split, re or im
 };
-
-template <int PREC>
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-  return tc_desc(addr, kLBO, Prec<PREC>::kSBO);
+constexpr uint32_t kHalfA = TM * 32;   // A's real (imaginary) parts of a chunk, one split
+constexpr uint32_t kBlockB = TN * 32;  // a block of B, one split
+// blocks of B (KIND 0: -Im, Re, Im; 1: Re and Im of each half's bands; 2: Re, -Im)
+__host__ __device__ constexpr uint32_t blocks_b(int kind) {
+  return kind == 0 ? 3 : (kind == 1 ? 4 : 2);
+}
+__host__ __device__ constexpr uint32_t stage_bytes(int kind) {
+  return 4 * kHalfA + 2 * blocks_b(kind) * kBlockB;
 }
 
-// byte offset of element (row r, real k kk) in a K-major no-swizzle tile
-template <int PREC>
-__device__ __forceinline__ int koff(int r, int kk) {
-  constexpr int pc = Prec<PREC>::kPerCore;
-  return (r >> 3) * (int)Prec<PREC>::kSBO + (kk / pc) * (int)kLBO + (r & 7) * 16 +
-         (kk % pc) * Prec<PREC>::kBytes;
-}
+__device__ __forceinline__ uint64_t sdesc(uint32_t addr) { return tc_desc(addr, kLBO, kSBO); }
 
 __device__ __forceinline__ float tf32_hi(float x) {
   uint32_t r;
@@ -90,28 +93,46 @@ __device__ __forceinline__ float tf32_hi(float x) {
   return __uint_as_float(r);
 }
 
-// x = hi + lo at byte offset off of the hi and lo tiles
-template <int PREC>
-__device__ __forceinline__ void put_split(char *hi, char *lo, int off, float x) {
-  if (PREC == 0) {
-    const float h = tf32_hi(x);
-    *(float *)(hi + off) = h;
-    *(float *)(lo + off) = x - h;
-  } else {
-    const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    *(__nv_bfloat16 *)(hi + off) = h;
-    *(__nv_bfloat16 *)(lo + off) = __float2bfloat16_rn(x - __bfloat162float(h));
+// N consecutive k of a row, split into hi and lo words
+template <int PREC, int N>
+struct Run {
+  static constexpr int kWords = PREC ? N / 2 : N;
+  uint32_t hi[kWords], lo[kWords];
+  __device__ __forceinline__ explicit Run(const float (&x)[N]) {
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+      if constexpr (PREC == 0) {
+        const float h = tf32_hi(x[j]);
+        hi[j] = __float_as_uint(h);
+        lo[j] = __float_as_uint(x[j] - h);
+      } else {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+        const float2 f = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(x[2 * j] - f.x, x[2 * j + 1] - f.y);
+        hi[j] = *(const uint32_t *)&h;
+        lo[j] = *(const uint32_t *)&l;
+      }
+    }
   }
-}
-
-// Two consecutive-k values as BF16 hi and lo halves, one 4-byte word each
-// (off 4-byte aligned: k even).
-__device__ __forceinline__ void put_split2(char *hi, char *lo, int off, float x0, float x1) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-  const float2 hf = __bfloat1622float2(h);
-  *(__nv_bfloat162 *)(hi + off) = h;
-  *(__nv_bfloat162 *)(lo + off) = __floats2bfloat162_rn(x0 - hf.x, x1 - hf.y);
-}
+  __device__ __forceinline__ void negate() {
+    constexpr uint32_t sign = PREC ? 0x80008000u : 0x80000000u;
+#pragma unroll
+    for (int j = 0; j < kWords; ++j) {
+      hi[j] ^= sign;
+      lo[j] ^= sign;
+    }
+  }
+  // a run is 16 (A) or 8 (B) bytes
+  __device__ __forceinline__ void put(char *at_hi, char *at_lo) const {
+    if constexpr (kWords == 4) {
+      *(uint4 *)at_hi = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *(uint4 *)at_lo = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    } else {
+      *(uint2 *)at_hi = make_uint2(hi[0], hi[1]);
+      *(uint2 *)at_lo = make_uint2(lo[0], lo[1]);
+    }
+  }
+};
 
 template <int PREC>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
@@ -144,35 +165,36 @@ __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t
 // The DFT kinds take their tile indices from blockIdx.x with the N tiles of
 // one M tile adjacent in launch order, so the M tile's inputs come from DRAM
 // once and from L2 for the other N tiles.
+//
+// Where A or B is one matrix for the whole batch (the spatial DFTs), the other
+// side's slices are one tall (fold: row m is row m mod slice_m of slice
+// m / slice_m) or, being contiguous, one wide matrix: tiles then cross slices, and
+// only the last one is padded.
 template <int OPB, int EPI, int PREC, int KIND = 0>
-// The forward DFT kind holds both cubes' next chunk in registers (152 of them
-// with 3xTF32) and runs one CTA per SM without spills; the others fit two.
-__global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm g, Dft3 f, int *err) {
+__global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *err) {
   extern __shared__ __align__(1024) char smem[];
   using P = Prec<PREC>;
   // two shared-memory stages, so that a chunk is staged while the previous
   // chunk's MMAs run, and two TMEM tiles (one per stage)
   constexpr uint32_t kCols = 256;
-  constexpr size_t kStageBytes = 2 * P::kTileA + 4 * P::kTileB;
+  constexpr uint32_t kStageBytes = stage_bytes(KIND), kLoB = blocks_b(KIND) * kBlockB;
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tslot;
-  __shared__ int s_ok;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int b = blockIdx.z;
   if (KIND == 0 && g.gate && !g.gate[b]) return;  // a gated-off batch entry (CTA-uniform)
-  const float2 *A = g.A + (size_t)b * g.sA;
-  const float2 *B = g.B + (size_t)b * g.sB;
-  float2 *C = g.C + (size_t)b * g.sC;
   int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
   // the DFT kinds: problem size, this batch entry's cubes
   int gM = g.M, gN = g.N, gK = g.K;
   const float *xb = nullptr, *yb = nullptr;
   const float2 *specb = nullptr;
-  if (KIND != 0) {
-    const int nt = ((KIND == 1 ? f.h : f.n3) + TN - 1) / TN;
+  if (KIND != 0 || g.fold) {
+    const int nt = ((KIND == 0 ? g.N : (KIND == 1 ? f.h : f.n3)) + TN - 1) / TN;
     m0 = (blockIdx.x / nt) * TM;
     n0 = (blockIdx.x % nt) * TN;
+  }
+  if (KIND != 0) {
     gM = (int)f.P;
     gN = KIND == 1 ? f.h : f.n3;
     gK = KIND == 1 ? f.n3 : f.h;
@@ -194,7 +216,6 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[0])));
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[1])));
     asm volatile("fence.mbarrier_init.release.cluster;");
-    s_ok = 1;
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -226,205 +247,178 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
     accRe[c] = 0.f;
     accIm[c] = 0.f;
   }
-  constexpr int TK = P::kTK, KR = P::kKR;
+  constexpr int TK = P::kTK, KR = P::kKR, kRun = P::kRun, kHalf = kRun / 2;
   // a chunk is TK complex K (KIND 0, 2) or KR real bands (KIND 1)
-  const int nchunks = KIND == 1 ? (gK + KR - 1) / KR : (gK + TK - 1) / TK;
+  constexpr int kStep = KIND == 1 ? KR : TK;
+  const int nchunks = (gK + kStep - 1) / kStep;
   // Staging is software-pipelined: chunk ch + 1's operands are loaded from
   // global memory into registers while chunk ch's MMAs run, then split and
   // stored to shared memory once those MMAs are done with the tiles.
-  // A tile: rows m0..m0+127, complex k0..k0+TK-1 -> real kk = k (re), k + TK
-  // (im).  Element e of a tile: a warp covers 8 rows x 4 k, so its 32 stores
-  // hit 32 distinct banks of a core-matrix row group and its loads are four
-  // 64-byte runs of a column.  B tiles (output columns n0..n0+63): row n holds
-  // op(B)(k, n) over k, 8 rows n x 4 k per warp (loads are runs of 4 k,
-  // B(k, n) at k + ldb n, or of 8 n, B(n, k) at n + ldb k).
-  constexpr int kPa = TM * TK / kThreads, kPb = TN * TK / kThreads;
-  float2 ra[kPa], rb[kPb] = {};
+  // A: this thread's row and its run of kRun k (KIND 1: of two runs of bands, TK
+  // apart, the halves of a chunk).  A warp loads 32 rows of one k and stores four
+  // contiguous core matrices.
+  const int ar = tid & (TM - 1), ak = (tid / TM) * kRun, am = m0 + ar;
+  const uint32_t aoff = (ar >> 3) * kSBO + (tid / TM) * kLBO + (ar & 7) * 16;
+  // B: its column n and its half run of k; a warp loads 8 columns by the chunk's
+  // K (whole sectors in either order), and half a warp stores one core matrix
+  const int bp = (lane & 1) | ((lane >> 4) << 1), br = 8 * warp + ((lane >> 1) & 7);
+  const int bk = bp * kHalf, bn = n0 + br;
+  const uint32_t boff = (br >> 3) * kSBO + (bp >> 1) * kLBO + (br & 7) * 16 + (bp & 1) * 8;
+  // the slice and the row in it of row m (KIND 0)
+  auto slice_of = [&](int m) -> int { return g.fold ? m / g.slice_m : b; };
+  auto row_of = [&](int m) -> int { return g.fold ? m % g.slice_m : m; };
+  // where the row's and the column's k = 0 are, the step along k, and the end of k
+  // (0: a row or column outside); 32-bit element steps, 64-bit addresses
+  const float2 *ap = nullptr, *bq = nullptr;
+  const float *xp = nullptr, *yp = nullptr;
+  size_t as = 1, bs = 1;
+  const int aend = am < gM ? gK : 0;
+  int bend = bn < gN ? gK : 0;
+  if (KIND == 0) {
+    const int m = am < gM ? am : 0, n = bn < gN ? bn : 0;
+    const float2 *A = g.A + (size_t)slice_of(m) * g.sA, *B = g.B + (size_t)b * g.sB;
+    as = OPB == 2 ? 1 : (size_t)g.lda;
+    ap = A + (OPB == 2 ? (size_t)g.lda * row_of(m) : (size_t)row_of(m)) + as * ak;
+    bs = OPB == 1 ? (size_t)g.ldb : 1;
+    bq = B + (OPB == 1 ? (size_t)n : (size_t)g.ldb * n) + bs * bk;
+  } else {
+    as = f.P;
+    const int m = am < gM ? am : 0;
+    if (KIND == 1) {
+      xp = xb + m + as * ak;
+      if (yb) yp = yb + m + as * ak;
+    } else {
+      ap = specb + wpos(m) + as * ak;
+    }
+  }
+  // The DFT kinds' B operand, twiddles exp(-2 pi i j / n3) from a table that stays
+  // in L1, is read when the chunk is stored.  Entry k of column n is j = n k mod n3:
+  // ti is this thread's first of the chunk, and j goes on by n, ti by n kStep.
+  unsigned ti = 0, tstep = 0, thalf = 0;
+  if (KIND != 0) {
+    const unsigned n3 = (unsigned)f.n3, n = (unsigned)bn;
+    ti = n * (unsigned)bk % n3;
+    tstep = n * (unsigned)kStep % n3;
+    thalf = n * (unsigned)TK % n3;
+  }
+  auto on = [&](unsigned j, unsigned by) -> unsigned {  // (j + by) mod n3, both below n3
+    j += by;
+    return j >= (unsigned)f.n3 ? j - (unsigned)f.n3 : j;
+  };
+  float2 ra[kRun], rb[KIND == 0 ? kHalf : 1];
   // KIND 1 with a second cube: its raw values, combined (x - ycoef y) only when
-  // the chunk is stored, so that the loads stay in flight meanwhile.  The DFT
-  // kinds' B operand (twiddles from a table of n3 entries that stays in L1) is
-  // read when the chunk is stored, not held in registers across the pipeline.
-  float2 ry[KIND == 1 ? kPa : 1] = {};
-  // 3xBF16: a thread takes two consecutive k of one row (items i, i + 1 with
-  // i even), so that each hi or lo store is one 4-byte word of two halves and
-  // a warp's 32 words (8 rows x 4 k pairs) again fall in 32 distinct banks
-  auto a_pos = [&](int i, int &r, int &kc) {
-    const int e = tid + kThreads * (PREC ? i >> 1 : i), rest = e >> 5;
-    r = ((rest % (TM / 8)) << 3) | ((e >> 2) & 7);
-    kc = ((rest / (TM / 8)) << 2) | (e & 3);
-    if (PREC) kc = (kc << 1) | (i & 1);
-  };
-  auto b_pos = [&](int i, int &n, int &kc) {
-    const int e = tid + kThreads * (PREC ? i >> 1 : i), rest = e >> 5;
-    n = ((rest % (TN / 8)) << 3) | ((e >> 2) & 7);
-    kc = ((rest / (TN / 8)) << 2) | (e & 3);
-    if (PREC) kc = (kc << 1) | (i & 1);
-  };
-  // the raw value of cube q at pixel gm, band c (0 outside the cube)
-  auto cval = [&](const float *q, int gm, int c) -> float {
-    return (gm < gM && c < gK) ? q[(size_t)gm + f.P * c] : 0.0f;
-  };
-  // exp(-2 pi i k c / n3) (0 outside the half spectrum or the bands)
-  auto twid = [&](int k, int c) -> float2 {
-    if (k >= f.h || c >= f.n3) return make_float2(0.f, 0.f);
-    return f.tw3[(unsigned)(k * c) % (unsigned)f.n3];
-  };
+  // the chunk is stored, so that the loads stay in flight meanwhile
+  float2 ry[KIND == 1 ? kRun : 1];
   auto load_chunk = [&](int k0) {
     if constexpr (KIND == 1) {
+      auto pair = [&](const float *q, int i) -> float2 {
+        const int k = k0 + ak + i;
+        return make_float2(k < aend ? q[as * (k0 + i)] : 0.f,
+                           k + TK < aend ? q[as * (k0 + TK + i)] : 0.f);
+      };
 #pragma unroll
-      for (int i = 0; i < kPa; ++i) {
-        int r, kc;
-        a_pos(i, r, kc);
-        ra[i] = make_float2(cval(xb, m0 + r, k0 + kc), cval(xb, m0 + r, k0 + TK + kc));
-        if (yb)
-          ry[KIND == 1 ? i : 0] =
-              make_float2(cval(yb, m0 + r, k0 + kc), cval(yb, m0 + r, k0 + TK + kc));
+      for (int i = 0; i < kRun; ++i) {
+        ra[i] = pair(xp, i);
+        if (yp) ry[KIND == 1 ? i : 0] = pair(yp, i);
       }
     } else {
+      const float2 *q = ap + as * k0;
 #pragma unroll
-      for (int i = 0; i < kPa; ++i) {
-        int r, kc;
-        a_pos(i, r, kc);
-        const int gm = m0 + r, gk = k0 + kc;
-        if (KIND == 2) {  // raw; conjugated (transposed slices) when stored
-          ra[i] = (gm < gM && gk < gK) ? specb[wpos(gm) + f.P * gk] : make_float2(0.f, 0.f);
-        } else if (OPB == 2) {  // A^H(m, k) = conj A(k, m): conjugated when stored
-          ra[i] = (gm < g.M && gk < g.K) ? A[gk + (size_t)g.lda * gm] : make_float2(0.f, 0.f);
-        } else {
-          ra[i] = (gm < g.M && gk < g.K) ? A[gm + (size_t)g.lda * gk] : make_float2(0.f, 0.f);
-        }
-      }
-      if (KIND == 0) {
+      for (int i = 0; i < kRun; ++i)  // raw: conjugated (OPB 2, transposed slices) when stored
+        ra[i] = k0 + ak + i < aend ? q[as * i] : make_float2(0.f, 0.f);
+      if constexpr (KIND == 0) {
+        const float2 *p = bq + bs * k0;
 #pragma unroll
-        for (int i = 0; i < kPb; ++i) {
-          int n, kc;
-          b_pos(i, n, kc);
-          const int gn = n0 + n, gk = k0 + kc;
-          // raw (OPB 1: conjugated when stored): combining a value where it is
-          // loaded makes the thread wait for it there
-          rb[i] = (gn < g.N && gk < g.K)
-                      ? (OPB != 1 ? B[gk + (size_t)g.ldb * gn] : B[gn + (size_t)g.ldb * gk])
-                      : make_float2(0.f, 0.f);
-        }
-      }
-    }
-  };
-  // B item i of the chunk at k0: (v, w) = KIND 0 the loaded op(B) value (w
-  // unused); KIND 1 the twiddles of bands k0 + kc and k0 + TK + kc; KIND 2
-  // w_k exp(+2 pi i k c / n3) of frequency k0 + kc (w unused)
-  auto bval = [&](int i, int k0, float2 &v, float2 &w) {
-    int n, kc;
-    b_pos(i, n, kc);
-    if (KIND == 0) {
-      v = rb[i];
-      if (OPB == 1) v.y = -v.y;
-    } else if (KIND == 1) {
-      v = twid(n0 + n, k0 + kc);
-      w = twid(n0 + n, k0 + TK + kc);
-    } else {
-      const int gn = n0 + n, gk = k0 + kc;
-      v = make_float2(0.f, 0.f);
-      if (gn < gN && gk < gK) {
-        const float2 t = f.tw3[(unsigned)(gk * gn) % (unsigned)f.n3];
-        const float wk = (gk == 0 || 2 * gk == f.n3) ? 1.0f : 2.0f;
-        v = make_float2(wk * t.x, -wk * t.y);
+        for (int i = 0; i < kHalf; ++i)  // raw (OPB 1: conjugated when stored): combining a
+          // value where it is loaded makes the thread wait for it there
+          rb[i] = k0 + bk + i < bend ? p[bs * i] : make_float2(0.f, 0.f);
       }
     }
   };
   // split the registers' chunk into the hi / lo tiles of stage `st`
   auto store_chunk = [&](int st, int k0) {
-    char *aHi = smem + st * kStageBytes, *aLo = aHi + P::kTileA;
-    // [Re | Im] B tiles of each split adjacent: one 128-row B operand
-    char *bReHi = aLo + P::kTileA, *bImHi = bReHi + P::kTileB;
-    char *bReLo = bImHi + P::kTileB, *bImLo = bReLo + P::kTileB;
-    // the A values as the MMAs take them: KIND 1 x - ycoef y, KIND 2 the
-    // conjugate on transposed slices
-    auto aval = [&](int i) -> float2 {
+    char *a = smem + st * kStageBytes + aoff, *q = smem + st * kStageBytes + 4 * kHalfA + boff;
+    float re[kRun], im[kRun];
+#pragma unroll
+    for (int i = 0; i < kRun; ++i) {
       float2 v = ra[i];
-      if (KIND == 1 && yb) {
+      if (KIND == 1 && yp) {
         const float2 w = ry[KIND == 1 ? i : 0];
         v = make_float2(v.x - f.ycoef * w.x, v.y - f.ycoef * w.y);
       }
       if ((KIND == 2 && f.trans) || (KIND == 0 && OPB == 2)) v.y = -v.y;
-      return v;
+      re[i] = v.x;
+      im[i] = v.y;
+    }
+    Run<PREC, kRun>(re).put(a, a + 2 * kHalfA);
+    Run<PREC, kRun>(im).put(a + kHalfA, a + 3 * kHalfA);
+    auto block = [&](int i, const Run<PREC, kHalf> &x) {
+      x.put(q + i * kBlockB, q + kLoB + i * kBlockB);
     };
-    if (PREC == 0) {
+    float u[kHalf], v[kHalf];
+    if constexpr (KIND == 0) {
 #pragma unroll
-      for (int i = 0; i < kPa; ++i) {
-        int r, kc;
-        a_pos(i, r, kc);
-        const float2 v = aval(i);
-        put_split<PREC>(aHi, aLo, koff<PREC>(r, kc), v.x);
-        put_split<PREC>(aHi, aLo, koff<PREC>(r, kc + TK), v.y);
+      for (int i = 0; i < kHalf; ++i) {
+        u[i] = rb[i].x;
+        v[i] = OPB == 1 ? -rb[i].y : rb[i].y;
       }
+      block(1, Run<PREC, kHalf>(u));
+      Run<PREC, kHalf> y(v);
+      block(2, y);
+      y.negate();
+      block(0, y);
+    } else if constexpr (KIND == 1) {
+      // the twiddles of the chunk's bands, half by half
 #pragma unroll
-      for (int i = 0; i < kPb; ++i) {
-        int n, kc;
-        b_pos(i, n, kc);
-        float2 v, w;
-        bval(i, k0, v, w);
-        if (KIND == 1) {  // real and imaginary twiddle parts of the chunk's bands
-          put_split<PREC>(bReHi, bReLo, koff<PREC>(n, kc), v.x);
-          put_split<PREC>(bReHi, bReLo, koff<PREC>(n, kc + TK), w.x);
-          put_split<PREC>(bImHi, bImLo, koff<PREC>(n, kc), v.y);
-          put_split<PREC>(bImHi, bImLo, koff<PREC>(n, kc + TK), w.y);
-          continue;
+      for (int h = 0; h < 2; ++h) {
+        unsigned j = h ? on(ti, thalf) : ti;
+#pragma unroll
+        for (int i = 0; i < kHalf; ++i) {
+          const float2 t = k0 + bk + h * TK + i < bend ? f.tw3[j] : make_float2(0.f, 0.f);
+          u[i] = t.x;
+          v[i] = t.y;
+          j = on(j, (unsigned)bn);
         }
-        put_split<PREC>(bReHi, bReLo, koff<PREC>(n, kc), v.x);  // [Re B | -Im B]
-        put_split<PREC>(bReHi, bReLo, koff<PREC>(n, kc + TK), -v.y);
-        if (KIND == 2) continue;  // Re C only
-        put_split<PREC>(bImHi, bImLo, koff<PREC>(n, kc), v.y);  // [Im B | Re B]
-        put_split<PREC>(bImHi, bImLo, koff<PREC>(n, kc + TK), v.x);
+        block(2 * h, Run<PREC, kHalf>(u));
+        block(2 * h + 1, Run<PREC, kHalf>(v));
       }
+      ti = on(ti, tstep);
     } else {
+      // w_k exp(+2 pi i k c / n3) of the chunk's frequencies, its imaginary part
+      // negated: the table's, as it is
+      unsigned j = ti;
 #pragma unroll
-      for (int i = 0; i < kPa; i += 2) {  // k pairs (kc even, kc + 1)
-        int r, kc;
-        a_pos(i, r, kc);
-        const float2 v0 = aval(i), v1 = aval(i + 1);
-        put_split2(aHi, aLo, koff<PREC>(r, kc), v0.x, v1.x);
-        put_split2(aHi, aLo, koff<PREC>(r, kc + TK), v0.y, v1.y);
+      for (int i = 0; i < kHalf; ++i) {
+        const int k = k0 + bk + i;
+        const float2 t = k < bend ? f.tw3[j] : make_float2(0.f, 0.f);
+        const float wk = (k == 0 || 2 * k == f.n3) ? 1.0f : 2.0f;
+        u[i] = wk * t.x;
+        v[i] = wk * t.y;
+        j = on(j, (unsigned)bn);
       }
-#pragma unroll
-      for (int i = 0; i < kPb; i += 2) {
-        int n, kc;
-        b_pos(i, n, kc);
-        float2 v0, v1, w0, w1;
-        bval(i, k0, v0, w0);
-        bval(i + 1, k0, v1, w1);
-        if (KIND == 1) {
-          put_split2(bReHi, bReLo, koff<PREC>(n, kc), v0.x, v1.x);
-          put_split2(bReHi, bReLo, koff<PREC>(n, kc + TK), w0.x, w1.x);
-          put_split2(bImHi, bImLo, koff<PREC>(n, kc), v0.y, v1.y);
-          put_split2(bImHi, bImLo, koff<PREC>(n, kc + TK), w0.y, w1.y);
-          continue;
-        }
-        put_split2(bReHi, bReLo, koff<PREC>(n, kc), v0.x, v1.x);  // [Re B | -Im B]
-        put_split2(bReHi, bReLo, koff<PREC>(n, kc + TK), -v0.y, -v1.y);
-        if (KIND == 2) continue;  // Re C only
-        put_split2(bImHi, bImLo, koff<PREC>(n, kc), v0.y, v1.y);  // [Im B | Re B]
-        put_split2(bImHi, bImLo, koff<PREC>(n, kc + TK), v0.x, v1.x);
-      }
+      block(0, Run<PREC, kHalf>(u));
+      block(1, Run<PREC, kHalf>(v));
+      ti = on(ti, tstep);
     }
   };
   // one thread: the chunk's MMAs on stage `st` into a fresh TMEM tile `st`,
   // committed to barrier `st`
   auto issue = [&](int st) {
-    const char *base = smem + st * kStageBytes;
-    const uint32_t a_hi = smem_u32(base), a_lo = a_hi + (uint32_t)P::kTileA;
-    const uint32_t b_hi = a_lo + (uint32_t)P::kTileA, b_lo = b_hi + 2 * (uint32_t)P::kTileB;
+    const uint32_t a = smem_u32(smem + st * kStageBytes), q = a + 4 * kHalfA;
     const uint32_t dt = tmem + (uint32_t)st * (2 * TN);
 #pragma unroll
-    for (int j = 0; j < KR / P::kMmaK; ++j) {  // one instruction spans two core matrices
-      const uint32_t ko = (uint32_t)j * 2 * kLBO;
+    for (int j = 0; j < 2; ++j) {  // A's real parts (KIND 1: the first bands), then the others
       const uint32_t acc0 = j > 0 ? 1u : 0u;  // a fresh tile per chunk
       // Re C (tile columns 0..63) and Im C (64..127) from one N = 128 MMA over
-      // the adjacent [Re | Im] B tiles, so that A is read once for both; the
-      // real part alone (KIND 2) from N = 64.  Three split products each.
+      // two adjacent blocks, so that A is read once for both; the real part alone
+      // (KIND 2) from N = 64.  Three split products each.
       const uint32_t id = KIND == 2 ? idesc : idesc2;
-      mma<PREC>(dt, sdesc<PREC>(a_hi + ko), sdesc<PREC>(b_hi + ko), id, acc0);
-      mma<PREC>(dt, sdesc<PREC>(a_hi + ko), sdesc<PREC>(b_lo + ko), id, 1u);
-      mma<PREC>(dt, sdesc<PREC>(a_lo + ko), sdesc<PREC>(b_hi + ko), id, 1u);
+      const uint64_t ah = sdesc(a + j * kHalfA), al = sdesc(a + (2 + j) * kHalfA);
+      const int blk = KIND == 0 ? 1 - j : (KIND == 1 ? 2 * j : j);
+      const uint64_t bh = sdesc(q + blk * kBlockB), bl = sdesc(q + kLoB + blk * kBlockB);
+      mma<PREC>(dt, ah, bh, id, acc0);
+      mma<PREC>(dt, ah, bl, id, 1u);
+      mma<PREC>(dt, al, bh, id, 1u);
     }
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -484,40 +478,37 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
       }
     } else {
       ok = false;
-      if (tid == 0) s_ok = 0;
     }
     asm volatile("tcgen05.fence::after_thread_sync;");
   };
+  // the stage is written and the tile drained by all; whether no wait ran out
   auto stage_barrier = [&]() {
     asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+    ok = __syncthreads_and(ok) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;");
   };
   if (nchunks > 0) load_chunk(0);
   // chunk ch: stage s = ch & 1 is written while chunk ch - 1's MMAs (stage
-  // s ^ 1) run; once those are done, chunk ch's MMAs are issued and chunk
-  // ch - 1's tile is drained while they run
-  for (int ch = 0; ch < nchunks && ok; ++ch) {
+  // s ^ 1) run; chunk ch's are queued behind them, and chunk ch - 1's tile is
+  // drained while they run
+  for (int ch = 0; ch < nchunks; ++ch) {
     const int st = ch & 1;
-    store_chunk(st, ch * (KIND == 1 ? KR : TK));  // stage st was last read by chunk ch - 2
-    if (ch + 1 < nchunks) load_chunk((ch + 1) * (KIND == 1 ? KR : TK));
+    store_chunk(st, ch * kStep);  // stage st was last read by chunk ch - 2
+    if (ch + 1 < nchunks) load_chunk((ch + 1) * kStep);
     stage_barrier();
-    if (ch > 0) {
-      wait_mmas(st ^ 1);
-      __syncthreads();
-      ok = ok && s_ok;
-      if (!ok) break;
-    }
+    if (!ok) break;
     if (tid == 0) issue(st);
     mark_issued(st);
-    if (ch > 0) drain(st ^ 1);
+    if (ch > 0) {
+      wait_mmas(st ^ 1);
+      if (ok) drain(st ^ 1);
+    }
   }
-  if (ok && nchunks > 0) {
+  if (nchunks > 0) {
     const int last = (nchunks - 1) & 1;
-    wait_mmas(last);
-    __syncthreads();
-    ok = ok && s_ok;
+    if (ok) wait_mmas(last);
+    ok = __syncthreads_and(ok) != 0;
     if (ok) drain(last);
   }
   if (!ok) {
@@ -529,7 +520,6 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
     // epilogue: thread (warp w, lane l) owns row m0 + 32 (w mod 4) + l of the
     // tile, columns colh .. colh + 31
     const int gm = m0 + row;
-    const int lb = g.lam3_period > 0 ? b % g.lam3_period : b;
     if (KIND == 1 && gm < gM) {
       float2 *ob = f.spec_out + (size_t)b * f.h * f.P + wpos(gm);
 #pragma unroll
@@ -568,18 +558,21 @@ __global__ void __launch_bounds__(kThreads, KIND == 1 ? 1 : 2) k_cgemm_tc(CGemm 
         }
       }
     } else if (KIND == 0 && gm < g.M) {
+      const int sl = slice_of(gm), mr = row_of(gm);
+      const int lb = g.lam3_period > 0 ? sl % g.lam3_period : sl;
+      float2 *C = g.C + (size_t)sl * g.sC + mr;
 #pragma unroll
       for (int c = 0; c < TN / 2; ++c) {
         const int n = n0 + colh + c;
         if (n >= g.N) break;
         float2 v = make_float2(accRe[c], accIm[c]);
         if (EPI == 1) {
-          const float den = g.mu * (1.0f + g.lam1[gm] + g.lam2[n] + g.lam3[lb]);
+          const float den = g.mu * (1.0f + g.lam1[mr] + g.lam2[n] + g.lam3[lb]);
           const float q = g.scale / den;
           v.x *= q;
           v.y *= q;
         }
-        C[gm + (size_t)g.ldc * n] = v;
+        C[(size_t)g.ldc * n] = v;
       }
     }
   }
@@ -666,8 +659,8 @@ __global__ void __launch_bounds__(128, 1) k_mma_peak(long long n_mma, int *err) 
                          ((uint32_t)(kProbeN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
   const uint32_t bar = smem_u32(&mbar);
   if (tid == 0) {
-    const uint64_t a = sdesc<PREC>(smem_u32(smem));
-    const uint64_t b = sdesc<PREC>(smem_u32(smem + (size_t)TM * P::kKR * P::kBytes));
+    const uint64_t a = sdesc(smem_u32(smem));
+    const uint64_t b = sdesc(smem_u32(smem + (size_t)TM * P::kKR * P::kBytes));
     for (long long i = 0; i < n_mma; ++i)
       mma<PREC>(tmem + (uint32_t)(i & 1) * kProbeN, a, b, idesc, i > 1 ? 1u : 0u);
     asm volatile(
@@ -681,25 +674,37 @@ __global__ void __launch_bounds__(128, 1) k_mma_peak(long long n_mma, int *err) 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-template <int PREC>
-size_t smem_bytes() {
-  return 2 * (2 * Prec<PREC>::kTileA + 4 * Prec<PREC>::kTileB);
-}
-
 template <int OPB, int EPI, int PREC>
-cudaError_t launch_one(const CGemm &g, int *err, cudaStream_t st) {
-  const size_t smem = smem_bytes<PREC>();
+cudaError_t launch_one(CGemm g, int *err, cudaStream_t st) {
+  const size_t smem = 2 * stage_bytes(0);
   cudaError_t e = cudaFuncSetAttribute(k_cgemm_tc<OPB, EPI, PREC>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((g.M + TM - 1) / TM, (g.N + TN - 1) / TN, g.batch);
+  // Slices that share A or B are one matrix, see the kernel (41 slices of 200 x 200,
+  // where 328 tiles left 24 to a second wave: 54 -> 31 us, wide, and 32, tall)
+  const long long rows = (long long)g.M * g.batch, cols = (long long)g.N * g.batch;
+  g.fold = 0;
+  if (OPB == 0 && g.batch > 1 && !g.gate && rows < (1 << 30) && cols < (1 << 21)) {
+    if (g.sB == 0) {
+      g.fold = 1;
+      g.slice_m = g.M;
+      g.M = (int)rows;
+      g.batch = 1;
+    } else if (EPI == 0 && g.sA == 0 && g.sB == (long long)g.ldb * g.N &&
+               g.sC == (long long)g.ldc * g.N) {
+      g.N = (int)cols;
+      g.batch = 1;
+    }
+  }
+  const unsigned mt = (g.M + TM - 1) / TM, nt = (g.N + TN - 1) / TN;
+  const dim3 grid = g.fold ? dim3(mt * nt) : dim3(mt, nt, g.batch);
   k_cgemm_tc<OPB, EPI, PREC><<<grid, kThreads, smem, st>>>(g, Dft3{}, err);
   return cudaGetLastError();
 }
 
 template <int KIND, int PREC>
 cudaError_t launch_dft(const Dft3 &f, int nb, int *err, cudaStream_t st) {
-  const size_t smem = smem_bytes<PREC>();
+  const size_t smem = 2 * stage_bytes(KIND);
   cudaError_t e = cudaFuncSetAttribute(k_cgemm_tc<0, 0, PREC, KIND>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -723,8 +728,6 @@ cudaError_t launch_prec(const CGemm &g, int *err, cudaStream_t st) {
 }
 
 }  // namespace
-
-size_t cgemm_tc_smem() { return smem_bytes<0>(); }
 
 long long cgemm_tc_wait_limit() { return kWaitLimit; }
 
