@@ -41,7 +41,9 @@
 // run goes to shared memory in one store.  With an element's position worked
 // out at a time and 4-byte stores, 123 slices of 200 x 200 took 114 us instead
 // of 105 (3xTF32; 288 of 256 x 256 with 3xBF16 249 instead of 200), and the
-// forward DFT of three 200 x 200 x 80 cubes 71 instead of 41.
+// forward DFT of three 200 x 200 x 80 cubes 71 instead of 41; sums in pairs and
+// TF32 by integers made the 105 95.  More chunks under way (asynchronous copies
+// into shared memory, read back) were slower: 110-123.
 // Two stages and two TMEM tiles pipeline the chunks: chunk k is loaded and
 // staged while chunk k - 1's MMAs run, and chunk k - 1's tile is drained while
 // chunk k's MMAs run.
@@ -87,10 +89,18 @@ __host__ __device__ constexpr uint32_t stage_bytes(int kind) {
 
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) { return tc_desc(addr, kLBO, kSBO); }
 
+// x to TF32, to nearest, ties away from zero: the value of cvt.rna.tf32.f32, which
+// takes five instructions here (a NaN may become an infinity: x - hi is NaN then)
 __device__ __forceinline__ float tf32_hi(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
+  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+}
+
+// two FP32 sums in one instruction, each rounded as alone
+__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1) {
+  asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n"
+      " add.rn.f32x2 a, a, b;\n mov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1)
+      : "f"(b0), "f"(b1));
 }
 
 // N consecutive k of a row, split into hi and lo words
@@ -456,9 +466,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
             : "r"(tl + tile + TN + c0));
       asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        if (KIND != 1) accRe[c0 + c] += __uint_as_float(re[c]);
-        if (KIND != 2) accIm[c0 + c] += __uint_as_float(im[c]);
+      for (int c = 0; c < 16; c += 2) {
+        if (KIND != 1)
+          add2(accRe[c0 + c], accRe[c0 + c + 1], __uint_as_float(re[c]),
+               __uint_as_float(re[c + 1]));
+        if (KIND == 1) {  // no packed pairs among this kind's live registers
+          accIm[c0 + c] += __uint_as_float(im[c]);
+          accIm[c0 + c + 1] += __uint_as_float(im[c + 1]);
+        } else if (KIND == 0) {
+          add2(accIm[c0 + c], accIm[c0 + c + 1], __uint_as_float(im[c]),
+               __uint_as_float(im[c + 1]));
+        }
       }
     }
     // the tile is rewritten only after every thread's reads
@@ -681,7 +699,7 @@ cudaError_t launch_one(CGemm g, int *err, cudaStream_t st) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // Slices that share A or B are one matrix, see the kernel (41 slices of 200 x 200,
-  // where 328 tiles left 24 to a second wave: 54 -> 31 us, wide, and 32, tall)
+  // where 328 tiles left 24 to a second wave: 54 -> 31 us)
   const long long rows = (long long)g.M * g.batch, cols = (long long)g.N * g.batch;
   g.fold = 0;
   if (OPB == 0 && g.batch > 1 && !g.gate && rows < (1 << 30) && cols < (1 << 21)) {
