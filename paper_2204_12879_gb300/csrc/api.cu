@@ -197,7 +197,9 @@ cudaError_t tsvt_post(const Dims &d, int nb, float *out, int mode, float *G4, co
   cudaError_t e;
   {
     Span sp(prof, LRSTV_K_CGEMM_E, st);
-    e = gemm(g, gs, st);
+    // the single operator's reconstruction keeps FP32 sums: 7 of its 1,000 us at
+    // 75 x 91 x 220, against an error that is the Jacobi's either way
+    e = gemm(g, gs.prec == 2 ? kSimt : gs, st);
   }
   if (e != cudaSuccess) return e;
   Span sp(prof, LRSTV_K_C2R_E, st);
@@ -1722,7 +1724,7 @@ int lrstv_zsolve(const float *T, int n1, int n2, int n3, const float w[3], float
   zsolve_ws(d, &tb, &A, &B, workspace);
   cudaStream_t st = (cudaStream_t)stream;
   CK(launch_tables(d, w, tb.tw3, tb.F1, tb.G1, tb.F2, tb.G2, tb.lam1, tb.lam2, tb.lam3, st));
-  CK(zsolve_core(d, 1, tb, T, mu, Z, A, B, st, nullptr, kSimt));
+  CK(zsolve_core(d, 1, tb, T, mu, Z, A, B, st, nullptr, kOperator));
   return LRSTV_OK;
 }
 
@@ -1742,7 +1744,7 @@ int lrstv_tsvt(const float *Ain, int n1, int n2, int n3, float t, float *out, vo
   cudaStream_t st = (cudaStream_t)stream;
   CK(launch_tw3(d.n3, tw, st));
   CK(tsvt_core(d, 1, Ain, nullptr, 0.0f, t, out, 0, nullptr, nullptr, 0.0f, 0, tw, A, B, V, sw,
-               st, nullptr, kSimt, nullptr, sched));
+               st, nullptr, kOperator, nullptr, sched));
   if (sweeps_host) {
     int *h = new (std::nothrow) int[d.h];
     if (!h) return LRSTV_ERR_ALLOC;

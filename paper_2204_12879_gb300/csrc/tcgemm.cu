@@ -15,6 +15,13 @@
 // drain into FP32 register accumulators: accumulation error then grows over
 // 16 terms, not over the whole K.
 //
+// The tensor core's truncation is then that of the hi*hi sums at each of the six
+// products.  prec = 2 forms a chunk's four small products first, so that only the
+// two hi*hi are added to a full-size sum: for the single operators, whose error
+// against FP64 this keeps below that of FP32 sums (Z-solve of 145 x 145 x 220:
+// 4.4e-7 relative, 8.9e-7 with prec = 0, 1.12e-6 with FP32 FMAs; 857 -> 281 us).  The iterations keep prec =
+// 0, whose rounding their runs' results have always had.
+//
 // Complex arithmetic as real GEMMs with K doubled: for a K chunk,
 //   Re C += [Re A | Im A] . [Re B | -Im B]^T,   Im C += [Re A | Im A] . [Im B | Re B]^T.
 //
@@ -71,11 +78,11 @@ constexpr uint32_t kLBO = 128, kSBO = 256;  // bytes
 // format (kind::tf32: TF32 = 2; kind::f16: BF16 = 1).
 template <int PREC>
 struct Prec {
-  static constexpr int kBytes = PREC ? 2 : 4;
+  static constexpr int kBytes = PREC == 1 ? 2 : 4;
   static constexpr int kTK = 32 / kBytes;   // complex K per chunk: 16 real terms per TMEM
   static constexpr int kKR = 2 * kTK;       // tile with 3xTF32
   static constexpr int kRun = 16 / kBytes;
-  static constexpr uint32_t kFmt = PREC ? 1u : 2u;
+  static constexpr uint32_t kFmt = PREC == 1 ? 1u : 2u;
 };
 constexpr uint32_t kHalfA = TM * 32;   // A's real (imaginary) parts of a chunk, one split
 constexpr uint32_t kBlockB = TN * 32;  // a block of B, one split
@@ -106,12 +113,12 @@ __device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1) {
 // N consecutive k of a row, split into hi and lo words
 template <int PREC, int N>
 struct Run {
-  static constexpr int kWords = PREC ? N / 2 : N;
+  static constexpr int kWords = PREC == 1 ? N / 2 : N;
   uint32_t hi[kWords], lo[kWords];
   __device__ __forceinline__ explicit Run(const float (&x)[N]) {
 #pragma unroll
     for (int j = 0; j < kWords; ++j) {
-      if constexpr (PREC == 0) {
+      if constexpr (PREC != 1) {
         const float h = tf32_hi(x[j]);
         hi[j] = __float_as_uint(h);
         lo[j] = __float_as_uint(x[j] - h);
@@ -125,7 +132,7 @@ struct Run {
     }
   }
   __device__ __forceinline__ void negate() {
-    constexpr uint32_t sign = PREC ? 0x80008000u : 0x80000000u;
+    constexpr uint32_t sign = PREC == 1 ? 0x80008000u : 0x80000000u;
 #pragma unroll
     for (int j = 0; j < kWords; ++j) {
       hi[j] ^= sign;
@@ -147,7 +154,7 @@ struct Run {
 template <int PREC>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                     uint32_t accumulate) {
-  if (PREC == 0)
+  if (PREC != 1)
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
@@ -416,19 +423,27 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
   auto issue = [&](int st) {
     const uint32_t a = smem_u32(smem + st * kStageBytes), q = a + 4 * kHalfA;
     const uint32_t dt = tmem + (uint32_t)st * (2 * TN);
+    // Re C (tile columns 0..63) and Im C (64..127) from one N = 128 MMA over two
+    // adjacent blocks, so that A is read once for both; the real part alone (KIND 2)
+    // from N = 64.  j: A's real parts (KIND 1: the first bands), then the others.
+    // Three split products each, into a fresh tile per chunk.
+    const uint32_t id = KIND == 2 ? idesc : idesc2;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {  // A's real parts (KIND 1: the first bands), then the others
-      const uint32_t acc0 = j > 0 ? 1u : 0u;  // a fresh tile per chunk
-      // Re C (tile columns 0..63) and Im C (64..127) from one N = 128 MMA over
-      // two adjacent blocks, so that A is read once for both; the real part alone
-      // (KIND 2) from N = 64.  Three split products each.
-      const uint32_t id = KIND == 2 ? idesc : idesc2;
+    for (int j = 0; j < 2; ++j) {
+      const uint32_t acc0 = j > 0 ? 1u : 0u;
       const uint64_t ah = sdesc(a + j * kHalfA), al = sdesc(a + (2 + j) * kHalfA);
       const int blk = KIND == 0 ? 1 - j : (KIND == 1 ? 2 * j : j);
       const uint64_t bh = sdesc(q + blk * kBlockB), bl = sdesc(q + kLoB + blk * kBlockB);
-      mma<PREC>(dt, ah, bh, id, acc0);
-      mma<PREC>(dt, ah, bl, id, 1u);
+      if (PREC != 2) mma<PREC>(dt, ah, bh, id, acc0);
+      mma<PREC>(dt, ah, bl, id, PREC != 2 ? 1u : acc0);
       mma<PREC>(dt, al, bh, id, 1u);
+    }
+    if (PREC == 2) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int blk = KIND == 0 ? 1 - j : (KIND == 1 ? 2 * j : j);
+        mma<PREC>(dt, sdesc(a + j * kHalfA), sdesc(q + blk * kBlockB), id, 1u);
+      }
     }
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -529,11 +544,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
     ok = __syncthreads_and(ok) != 0;
     if (ok) drain(last);
   }
-  if (!ok) {
-    if (tid == 0 && err) atomicExch(err, 1);
-    // give MMAs still in flight a last bounded chance to land before the free
+  // give MMAs still in flight a last bounded chance to land before the free
+  auto last_wait = [&]() {
     if (out0) mbar_wait(bar0, ph0);
     if (out1) mbar_wait(bar1, ph1);
+  };
+  if (PREC == 2 && !ok) {  // the single operators have no flag to set: the tile is not a number
+    last_wait();
+#pragma unroll
+    for (int c = 0; c < TN / 2; ++c) accRe[c] = accIm[c] = __int_as_float(0x7fffffff);
+  }
+  if (PREC != 2 && !ok) {
+    if (tid == 0 && err) atomicExch(err, 1);
+    last_wait();
   } else if (nchunks > 0) {
     // epilogue: thread (warp w, lane l) owns row m0 + 32 (w mod 4) + l of the
     // tile, columns colh .. colh + 31
@@ -736,7 +759,8 @@ cudaError_t launch_dft(const Dft3 &f, int nb, int *err, cudaStream_t st) {
 template <int PREC>
 cudaError_t launch_prec(const CGemm &g, int *err, cudaStream_t st) {
   if (g.opA == 1) {  // A^H B only
-    if (g.opB == 0 && g.epi == 0) return launch_one<2, 0, PREC>(g, err, st);
+    if constexpr (PREC != 2)
+      if (g.opB == 0 && g.epi == 0) return launch_one<2, 0, PREC>(g, err, st);
     return cudaErrorInvalidValue;
   }
   if (g.opB == 0 && g.epi == 0) return launch_one<0, 0, PREC>(g, err, st);
@@ -775,8 +799,14 @@ cudaError_t launch_mma_peak(int prec, int nsm, long long n_mma, int *err, cudaSt
 cudaError_t launch_dft3_tc(int kind, const Dft3 &f, int nb, int *err, cudaStream_t st, int prec) {
   if (f.P == 0 || nb <= 0) return cudaSuccess;
   if (f.P > (size_t)TM * 0x7fffffff / 4) return cudaErrorInvalidValue;
-  if (kind == 1) return prec ? launch_dft<1, 1>(f, nb, err, st) : launch_dft<1, 0>(f, nb, err, st);
-  if (kind == 2) return prec ? launch_dft<2, 1>(f, nb, err, st) : launch_dft<2, 0>(f, nb, err, st);
+  if (kind == 1)
+    return prec == 1   ? launch_dft<1, 1>(f, nb, err, st)
+           : prec == 2 ? launch_dft<1, 2>(f, nb, err, st)
+                       : launch_dft<1, 0>(f, nb, err, st);
+  if (kind == 2)
+    return prec == 1   ? launch_dft<2, 1>(f, nb, err, st)
+           : prec == 2 ? launch_dft<2, 2>(f, nb, err, st)
+                       : launch_dft<2, 0>(f, nb, err, st);
   return cudaErrorInvalidValue;
 }
 
@@ -785,6 +815,7 @@ cudaError_t launch_cgemm_tc(const CGemm &g, int *err, cudaStream_t st, int prec)
   if (g.epi == 2) return cudaErrorInvalidValue;  // SIMT kernel only
   if (prec == 0) return launch_prec<0>(g, err, st);
   if (prec == 1) return launch_prec<1>(g, err, st);
+  if (prec == 2) return launch_prec<2>(g, err, st);
   return cudaErrorInvalidValue;
 }
 

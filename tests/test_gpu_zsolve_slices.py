@@ -37,3 +37,20 @@ def test_tiles_across_slices(L, orc, shape, bf16):
     ref = orc.zsolve(T, mu, w)
     # 3xTF32 carries 2^-21 a term, 3xBF16 2^-17, through six unitary passes
     assert maxabs(got, ref) <= (2e-4 if bf16 else 1e-5) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("shape", SHAPES + [(145, 145, 66)])
+def test_single_operator_error(L, orc, shape):
+    """lrstv_zsolve on the tensor cores, its small split products summed first."""
+    T = f32(np.random.default_rng(sum(shape)).standard_normal(shape))
+    w = (1.0, 0.6, 1.4)
+    got = host(L.lrstv_zsolve(dev(T), shape, 0.7, w), shape)
+    ref = orc.zsolve(T, 0.7, w)
+    # a pass over K terms: the dropped lo*lo and two truncations of each chunk (3 x
+    # 2^-23), the sum of K / 8 chunks, rounded tables and results (2^-24 each); two
+    # passes a mode, of which each is unitary up to its scale
+    u = 2.0 ** -24
+    bound = sum(2 * (6 + np.ceil(k / 8) + 2) * u for k in shape)
+    err = np.linalg.norm(np.asarray(got, np.float64) - ref) / np.linalg.norm(ref)
+    print(shape, "error", err, "bound", bound)
+    assert err <= bound
