@@ -2,7 +2,9 @@
 // (arXiv 2204.12879, Section III-C): the fused L-update / T_z assembly, the
 // fused F / S / multiplier update, and the standalone difference operators.
 //
-// Thread mapping: one thread per (i, j) pixel column and a chunk of bands k;
+// Thread mapping of the fused updates where n1 is no multiple of four (the vector
+// forms and the operators have their own): one thread per (i, j) pixel column and
+// a chunk of bands k;
 // a warp spans 32 consecutive i (coalesced 128-byte rows).  Walking k inside
 // the thread keeps the mode-3 neighbour in a register, so each cube is read
 // once; the mode-1 / mode-2 neighbours come from L1 (the same block read
@@ -186,57 +188,86 @@ __global__ void __launch_bounds__(kBX *kBY)
   }
 }
 
-__global__ void __launch_bounds__(kBX *kBY)
-    k_diff(int n1, int n2, int n3, size_t N, int kchunk, const float *__restrict__ x, float w0,
-           float w1, float w2, float *__restrict__ g) {
-  const int i = blockIdx.x * kBX + threadIdx.x;
-  const int j = blockIdx.y * kBY + threadIdx.y;
-  if (i >= n1 || j >= n2) return;
-  const int k0 = blockIdx.z * kchunk;
-  const int k1 = min(n3, k0 + kchunk);
-  const size_t P = (size_t)n1 * n2;
-  const size_t col = (size_t)i + (size_t)n1 * j;
-  const size_t colp1 = (i == n1 - 1) ? col + 1 - n1 : col + 1;
-  const size_t colp2 = (j == n2 - 1) ? col - (size_t)n1 * (n2 - 1) : col + n1;
-  float xc = x[col + P * k0];
-  for (int k = k0; k < k1; ++k) {
-    const size_t v = col + P * k;
-    const int kp = (k == n3 - 1) ? 0 : k + 1;
-    const float x3 = x[col + P * kp];
-    g[v] = w0 * (x[colp1 + P * k] - xc);
-    g[v + N] = w1 * (x[colp2 + P * k] - xc);
-    g[v + 2 * N] = w2 * (x3 - xc);
-    xc = x3;
+// The difference operators, for any n1 (a row of 511 voxels starts at every
+// alignment, so that the loads stay single floats): memory-bound.  A thread has
+// kVox voxels of one band, a block 1,024 consecutive ones, and all loads are
+// issued before the first use; the bands' neighbours come from L2.  At 511 x 512 x
+// 191 the difference takes 138 us and its adjoint 153 (118 at the copy rate); one
+// column of bands a thread, one band after another, took 221 each, four bands at a
+// time 184 and 171; with 2, 6 and 8 voxels here 157, 164 and 277.
+constexpr int kVox = 4;
+
+__global__ void __launch_bounds__(256)
+    k_diff(int n1, int n2, int n3, size_t N, const float *__restrict__ x, float w0, float w1,
+           float w2, float *__restrict__ g) {
+  const int P = n1 * n2, k = blockIdx.y, c0 = blockIdx.x * (256 * kVox) + threadIdx.x;
+  const float *xk = x + (size_t)P * k, *xn = x + (size_t)P * (k == n3 - 1 ? 0 : k + 1);
+  g += (size_t)P * k;
+  float v[kVox], a[kVox], b[kVox], c[kVox];
+#pragma unroll
+  for (int u = 0; u < kVox; ++u) {
+    const int col = min(c0 + 256 * u, P - 1), j = col / n1, i = col - j * n1;
+    v[u] = xk[col];
+    a[u] = xk[i == n1 - 1 ? col + 1 - n1 : col + 1];
+    b[u] = xk[j == n2 - 1 ? i : col + n1];
+    c[u] = xn[col];
+  }
+#pragma unroll
+  for (int u = 0; u < kVox; ++u) {
+    const int col = c0 + 256 * u;
+    if (col >= P) break;
+    g[col] = w0 * (a[u] - v[u]);
+    g[col + N] = w1 * (b[u] - v[u]);
+    g[col + 2 * N] = w2 * (c[u] - v[u]);
   }
 }
 
-__global__ void __launch_bounds__(kBX *kBY)
-    k_diff_adjoint(int n1, int n2, int n3, size_t N, int kchunk, const float *__restrict__ g,
-                   float w0, float w1, float w2, float *__restrict__ x) {
-  const int i = blockIdx.x * kBX + threadIdx.x;
-  const int j = blockIdx.y * kBY + threadIdx.y;
-  if (i >= n1 || j >= n2) return;
-  const int k0 = blockIdx.z * kchunk;
-  const int k1 = min(n3, k0 + kchunk);
-  const size_t P = (size_t)n1 * n2;
-  const size_t col = (size_t)i + (size_t)n1 * j;
-  const size_t colm1 = (i == 0) ? col + n1 - 1 : col - 1;
-  const size_t colm2 = (j == 0) ? col + (size_t)n1 * (n2 - 1) : col - n1;
-  const float *g1 = g, *g2 = g + N, *g3 = g + 2 * N;
-  const int km = (k0 == 0) ? n3 - 1 : k0 - 1;
-  float g3prev = g3[col + P * km];
-  for (int k = k0; k < k1; ++k) {
-    const size_t v = col + P * k;
-    const float c3 = g3[v];
-    x[v] = w0 * (g1[colm1 + P * k] - g1[v]) + w1 * (g2[colm2 + P * k] - g2[v]) + w2 * (g3prev - c3);
-    g3prev = c3;
+__global__ void __launch_bounds__(256)
+    k_diff_adjoint(int n1, int n2, int n3, size_t N, const float *__restrict__ g, float w0,
+                   float w1, float w2, float *__restrict__ x) {
+  const int P = n1 * n2, k = blockIdx.y, c0 = blockIdx.x * (256 * kVox) + threadIdx.x;
+  const float *g1 = g + (size_t)P * k, *g2 = g1 + N, *g3 = g2 + N,
+              *gp = g + 2 * N + (size_t)P * (k == 0 ? n3 - 1 : k - 1);
+  x += (size_t)P * k;
+  float a[kVox], am[kVox], b[kVox], bm[kVox], c[kVox], cm[kVox];
+#pragma unroll
+  for (int u = 0; u < kVox; ++u) {
+    const int col = min(c0 + 256 * u, P - 1), j = col / n1, i = col - j * n1;
+    a[u] = g1[col];
+    am[u] = g1[i == 0 ? col + n1 - 1 : col - 1];
+    b[u] = g2[col];
+    bm[u] = g2[j == 0 ? i + n1 * (n2 - 1) : col - n1];
+    c[u] = g3[col];
+    cm[u] = gp[col];
+  }
+#pragma unroll
+  for (int u = 0; u < kVox; ++u) {
+    const int col = c0 + 256 * u;
+    if (col >= P) break;
+    x[col] = w0 * (am[u] - a[u]) + w1 * (bm[u] - b[u]) + w2 * (cm[u] - c[u]);
   }
 }
 
-__global__ void k_soft(const float *__restrict__ x, size_t n, float thr, float *__restrict__ y) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
-       e += (size_t)gridDim.x * blockDim.x)
-    y[e] = soft_thr(x[e], thr);
+// two float4 a thread (quads of them in all), or single floats where an array is
+// not 16-byte aligned and for the last n mod 4
+__global__ void __launch_bounds__(256)
+    k_soft(const float *__restrict__ x, size_t n, size_t quads, float thr,
+           float *__restrict__ y) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x,
+               all = gridDim.x * (size_t)blockDim.x;
+  const float4 *x4 = reinterpret_cast<const float4 *>(x);
+  float4 *y4 = reinterpret_cast<float4 *>(y);
+  auto thr4 = [&](float4 v) {
+    return make_float4(soft_thr(v.x, thr), soft_thr(v.y, thr), soft_thr(v.z, thr),
+                       soft_thr(v.w, thr));
+  };
+  for (size_t e = t; e < quads; e += 2 * all) {
+    const bool two = e + all < quads;
+    const float4 v = x4[e], u = two ? x4[e + all] : v;
+    y4[e] = thr4(v);
+    if (two) y4[e + all] = thr4(u);
+  }
+  for (size_t e = 4 * quads + t; e < n; e += all) y[e] = soft_thr(x[e], thr);
 }
 
 // ---------------------------------------------------------------------------
@@ -495,25 +526,27 @@ cudaError_t launch_fs_dual(const Dims &d, const float *Y, const float *L, const 
 
 cudaError_t launch_diff(const Dims &d, const float *x, const float w[3], float *g,
                         cudaStream_t st) {
-  Chunking c = chunking(d);
-  k_diff<<<c.grid, dim3(kBX, kBY), 0, st>>>(d.n1, d.n2, d.n3, d.N, c.kchunk, x, w[0], w[1], w[2],
+  const dim3 grid((unsigned)((d.P + 256 * kVox - 1) / (256 * kVox)), d.n3);
+  k_diff<<<grid, 256, 0, st>>>(d.n1, d.n2, d.n3, d.N, x, w[0], w[1], w[2],
                                             g);
   return cudaGetLastError();
 }
 
 cudaError_t launch_diff_adjoint(const Dims &d, const float *g, const float w[3], float *x,
                                 cudaStream_t st) {
-  Chunking c = chunking(d);
-  k_diff_adjoint<<<c.grid, dim3(kBX, kBY), 0, st>>>(d.n1, d.n2, d.n3, d.N, c.kchunk, g, w[0],
+  const dim3 grid((unsigned)((d.P + 256 * kVox - 1) / (256 * kVox)), d.n3);
+  k_diff_adjoint<<<grid, 256, 0, st>>>(d.n1, d.n2, d.n3, d.N, g, w[0],
                                                     w[1], w[2], x);
   return cudaGetLastError();
 }
 
 cudaError_t launch_soft(const float *x, size_t n, float thr, float *y, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  size_t blocks = (n + 255) / 256;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  k_soft<<<(unsigned)blocks, 256, 0, st>>>(x, n, thr, y);
+  const bool aligned = (((size_t)x | (size_t)y) & 15) == 0;
+  const size_t quads = aligned ? n / 4 : 0;
+  size_t blocks = ((aligned ? (n + 7) / 8 : n) + 255) / 256;
+  if (blocks > 152 * 1024) blocks = 152 * 1024;
+  k_soft<<<(unsigned)blocks, 256, 0, st>>>(x, n, quads, thr, y);
   return cudaGetLastError();
 }
 
