@@ -15,34 +15,48 @@ namespace lrstv {
 namespace {
 
 // ------------------------------------------------------------------ tables
-__global__ void k_dft_matrix(int n, float2 *__restrict__ F, float2 *__restrict__ G) {
-  const size_t total = (size_t)n * n;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const size_t a = e % n, t = e / n;
-    const size_t m = (a * t) % (size_t)n;
-    double s, c;
-    sincospi(2.0 * (double)m / (double)n, &s, &c);
-    F[e] = make_float2((float)c, (float)-s);  // exp(-2 pi i a t / n)
-    G[e] = make_float2((float)c, (float)s);   // exp(+2 pi i a t / n)
-  }
+__device__ __forceinline__ float2 twiddle(unsigned m, int n) {  // exp(-2 pi i m / n)
+  double s, c;
+  sincospi(2.0 * (double)m / (double)n, &s, &c);
+  return make_float2((float)c, (float)-s);
 }
 
 __global__ void k_tw3(int n3, float2 *__restrict__ tw) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n3; m += gridDim.x * blockDim.x) {
-    double s, c;
-    sincospi(2.0 * (double)m / (double)n3, &s, &c);
-    tw[m] = make_float2((float)c, (float)-s);
-  }
+  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n3; m += gridDim.x * blockDim.x)
+    tw[m] = twiddle(m, n3);
 }
 
-// lam[a] = w^2 |exp(2 pi i a / n) - 1|^2 = w^2 4 sin^2(pi a / n): the DFT
-// eigenvalues of w^2 D^T D for a circular forward difference of length n.
-__global__ void k_lam(int n, double w, float *__restrict__ lam) {
-  for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
-    const double s = sinpi((double)a / (double)n);
-    lam[a] = (float)(w * w * 4.0 * s * s);
+// All tables of a solve in one launch (six launches of 5 us each before, a tenth of
+// a Z-solve of 145 x 145 x 220).  Block row 0, 1: the DFT matrices of n1, n2 and
+// their conjugates; 2: the mode-3 twiddles and the eigenvalues lam[a] = w^2
+// |exp(2 pi i a / n) - 1|^2 = w^2 4 sin^2(pi a / n) of w^2 D^T D for circular
+// forward differences of length n.
+__global__ void k_tables(int n1, int n2, int n3, float w1, float w2, float w3,
+                         float2 *__restrict__ tw3, float2 *__restrict__ F1,
+                         float2 *__restrict__ G1, float2 *__restrict__ F2,
+                         float2 *__restrict__ G2, float *__restrict__ lam1,
+                         float *__restrict__ lam2, float *__restrict__ lam3) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+  if (blockIdx.y < 2) {
+    const unsigned n = blockIdx.y ? n2 : n1;
+    float2 *F = blockIdx.y ? F2 : F1, *G = blockIdx.y ? G2 : G1;
+    for (unsigned e = t; e < n * n; e += all) {
+      const float2 v = twiddle(e % n * (e / n) % n, n);
+      F[e] = v;                       // exp(-2 pi i a t / n)
+      G[e] = make_float2(v.x, -v.y);  // exp(+2 pi i a t / n)
+    }
+    return;
   }
+  for (unsigned m = t; m < n3; m += all) tw3[m] = twiddle(m, n3);
+  auto lam = [&](int n, double w, float *out) {
+    for (unsigned a = t; a < n; a += all) {
+      const double s = sinpi((double)a / (double)n);
+      out[a] = (float)(w * w * 4.0 * s * s);
+    }
+  };
+  lam(n1, w1, lam1);
+  lam(n2, w2, lam2);
+  lam(n3, w3, lam3);
 }
 
 // --------------------------------------------------------- mode-3 DFTs
@@ -329,14 +343,11 @@ cudaError_t launch_tw3(int n3, float2 *tw3, cudaStream_t st) {
 cudaError_t launch_tables(const Dims &d, const float w[3], float2 *tw3, float2 *F1, float2 *G1,
                           float2 *F2, float2 *G2, float *lam1, float *lam2, float *lam3,
                           cudaStream_t st) {
-  cudaError_t e = launch_tw3(d.n3, tw3, st);
-  if (e != cudaSuccess) return e;
-  auto blocks = [](size_t n) { return (unsigned)((n + 255) / 256 > 1024 ? 1024 : (n + 255) / 256); };
-  k_dft_matrix<<<blocks((size_t)d.n1 * d.n1), 256, 0, st>>>(d.n1, F1, G1);
-  k_dft_matrix<<<blocks((size_t)d.n2 * d.n2), 256, 0, st>>>(d.n2, F2, G2);
-  k_lam<<<blocks(d.n1), 256, 0, st>>>(d.n1, (double)w[0], lam1);
-  k_lam<<<blocks(d.n2), 256, 0, st>>>(d.n2, (double)w[1], lam2);
-  k_lam<<<blocks(d.n3), 256, 0, st>>>(d.n3, (double)w[2], lam3);
+  const int longest = d.n1 > d.n2 ? d.n1 : d.n2;
+  const size_t work = (size_t)longest * longest > d.n3 ? (size_t)longest * longest : d.n3;
+  const unsigned blocks = (unsigned)((work + 255) / 256 > 1024 ? 1024 : (work + 255) / 256);
+  k_tables<<<dim3(blocks, 3), 256, 0, st>>>(d.n1, d.n2, d.n3, w[0], w[1], w[2], tw3, F1, G1, F2, G2,
+                                            lam1, lam2, lam3);
   return cudaGetLastError();
 }
 
