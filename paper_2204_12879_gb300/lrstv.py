@@ -102,6 +102,7 @@ _P = ctypes.c_void_p
 _I = ctypes.c_int
 _F = ctypes.c_float
 _SZ = ctypes.c_size_t
+_Float3 = ctypes.c_float * 3
 # name -> argtypes (every entry point returns int status unless listed in _RESTYPE)
 _SIGS = {
     "lrstv_status_string": [_I],
@@ -193,23 +194,33 @@ def kernel_name(k: int) -> str:
 
 
 def _call(name, *args):
-    rc = getattr(load(), name)(*args)
+    rc = getattr(_lib or load(), name)(*args)
     if rc != 0:
         raise LrstvError(name, rc)
     return rc
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("liblrstv needs a CUDA device; there is no CPU path")
-    return torch
+    # asking the driver for devices took a fifth of a small operator's call, four
+    # times a call: asked until one was found
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("liblrstv needs a CUDA device; there is no CPU path")
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream(stream=None):
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    # the current stream's handle without a Stream object around it (3 us)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _dev(t, n=None):
@@ -223,7 +234,7 @@ def _dev(t, n=None):
 
 
 def _w(w):
-    return (ctypes.c_float * 3)(*[float(x) for x in w])
+    return _Float3(*[float(x) for x in w])
 
 
 def _empty(n, device=None):
