@@ -279,8 +279,18 @@ __global__ void __launch_bounds__(256)
 // pair checks.  One CTA; V is n x n column-major in global memory (the
 // identity is written when warm = 0); lam receives diag(B); *sweeps_out the
 // sweeps used, -max_sweeps at the cap.
+//
+// What bounds it: the latency of a round, n of them a sweep one after another.
+// Half of the warps rotate B; the other half rotate V, which decides nothing, a
+// round behind them: the lists of a round's pairs are in two copies, handed over
+// by named barriers.  A round in which no pair is rotated costs one barrier.  Ten
+// iterations on 64 x 60 x 31 took 30.4 ms with V in turn, 23.7 now (128 x 120 x 31,
+// six: 36.4, 29.9); V in shared memory made no difference.
 constexpr int kSyevjMax = 224;
 constexpr int kSyevjThreads = 1024;
+// the threads that rotate B (64 x 60 x 31: 256, 384 and 640 alike; 200 x 190 x 20: 15%,
+// 1% and 10% slower)
+constexpr int kSyevjB = 512;
 constexpr int kVBatch = 8;  // V items a thread has in flight
 
 size_t syevj_smem(int n) {
@@ -288,15 +298,36 @@ size_t syevj_smem(int n) {
   return sizeof(float) * (size_t)m * m;
 }
 
+// a round's pairs: all of them, the rotated ones and the others
+struct Pairs {
+  int p[kSyevjMax / 2], q[kSyevjMax / 2], go[kSyevjMax / 2];
+  float c[kSyevjMax / 2], s[kSyevjMax / 2], t[kSyevjMax / 2];
+  int rot[kSyevjMax / 2], still[kSyevjMax / 2];
+  int k;  // rotated pairs; -1: no round is left
+};
+
+// barriers of the threads that rotate B, and of all: pairs in copy i are ready
+// (V's threads wait), and V is done with them (B's threads wait)
+__device__ __forceinline__ void b_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kSyevjB) : "memory");
+}
+__device__ __forceinline__ void all_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kSyevjThreads) : "memory");
+}
+__device__ __forceinline__ void all_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kSyevjThreads) : "memory");
+}
+constexpr int kReady = 2, kDone = 4;  // + copy
+
 __global__ void __launch_bounds__(kSyevjThreads, 1)
     k_syevj(int n, const float *__restrict__ B0, float *__restrict__ V, int warm,
             float *__restrict__ lam, int max_sweeps, int *__restrict__ sweeps_out) {
   extern __shared__ float sB[];  // m x m, row-major
-  __shared__ int s_p[kSyevjMax / 2], s_q[kSyevjMax / 2], s_go[kSyevjMax / 2];
-  __shared__ float s_c[kSyevjMax / 2], s_s[kSyevjMax / 2], s_t[kSyevjMax / 2];
-  __shared__ int s_rot[kSyevjMax / 2], s_still[kSyevjMax / 2];  // rotated / other pairs
+  __shared__ Pairs s_pairs[2];
   __shared__ float s_red[32];
-  __shared__ int s_any, s_nrot, s_nstill, s_sweep_any;
+  // the lists' lengths, in three copies: a round counts in copy i, and clears copy
+  // i + 2 after its barrier
+  __shared__ int s_nrot[3], s_nstill[3];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = n + (n & 1), h = m / 2;
   const float eps = FLT_EPSILON * 0.5f;
@@ -309,6 +340,7 @@ __global__ void __launch_bounds__(kSyevjThreads, 1)
   }
   if (!warm)
     for (int e = tid; e < n * n; e += blockDim.x) V[e] = (e % n) == (e / n) ? 1.0f : 0.0f;
+  if (tid < 3) s_nrot[tid] = s_nstill[tid] = 0;
   float dmax = 0.0f;
   for (int i = tid; i < n; i += blockDim.x) dmax = fmaxf(dmax, fabsf(B0[i + (size_t)n * i]));
 #pragma unroll
@@ -324,26 +356,59 @@ __global__ void __launch_bounds__(kSyevjThreads, 1)
   __syncthreads();
   const float floor_abs = eps * s_red[0];
 
-  int sweeps = 0;
+  if (tid >= kSyevjB) {
+    // V := V J on the rotated pairs' columns (L2-resident): each thread loads a
+    // batch of its items before it stores any, so the loads' latencies overlap
+    constexpr int kVT = kSyevjThreads - kSyevjB;
+    for (int copy = 0;; copy ^= 1) {
+      all_sync(kReady + copy);
+      const Pairs &s = s_pairs[copy];
+      const int k = s.k;
+      if (k < 0) return;
+      for (int base = tid - kSyevjB; base < k * n; base += kVT * kVBatch) {
+        float vp[kVBatch], vq[kVBatch];
+        int ip[kVBatch], iq[kVBatch], pr[kVBatch];
+#pragma unroll
+        for (int u = 0; u < kVBatch; ++u) {
+          const int e = base + kVT * u;
+          pr[u] = -1;
+          if (e < k * n) {
+            const int P = s.rot[e / n], row = e % n;
+            pr[u] = P;
+            ip[u] = row + n * s.p[P];
+            iq[u] = row + n * s.q[P];
+            vp[u] = V[ip[u]];
+            vq[u] = V[iq[u]];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kVBatch; ++u) {
+          if (pr[u] < 0) continue;
+          const float c = s.c[pr[u]], sn = s.s[pr[u]];
+          V[ip[u]] = c * vp[u] - sn * vq[u];
+          V[iq[u]] = sn * vp[u] + c * vq[u];
+        }
+      }
+      all_arrive(kDone + copy);
+    }
+  }
+
+  int sweeps = 0, cnt = 0, copy = 0, used = 0;  // copy: the lists', used: rounds handed to V
   bool converged = n < 2;
   if (converged) sweeps = 1;
   for (int sweep = 1; sweep <= max_sweeps && !converged; ++sweep) {
-    if (tid == 0) s_sweep_any = 0;
+    bool any = false;
     for (int r = 0; r < m - 1; ++r) {
-      if (tid == 0) {
-        s_any = 0;
-        s_nrot = 0;
-        s_nstill = 0;
-      }
-      __syncthreads();
-      if (tid < h) {
+      Pairs &s = s_pairs[copy];
+      if (32 * warp < h) {
+        const bool in = tid < h;
         int p, q;
         if (tid == 0) {
           p = r;
           q = m - 1;
         } else {
           p = (r + tid) % (m - 1);
-          q = (r - tid + m - 1) % (m - 1);
+          q = (r - tid + 2 * (m - 1)) % (m - 1);
         }
         if (p > q) {
           const int x = p;
@@ -352,65 +417,83 @@ __global__ void __launch_bounds__(kSyevjThreads, 1)
         }
         int go = 0;
         float c = 1.0f, sn = 0.0f, t = 0.0f;
-        if (q < n) {
+        if (in && q < n) {
           const float app = sB[p * m + p], aqq = sB[q * m + q], apq = sB[p * m + q];
           const float aa = fabsf(apq);
-          if (aa > floor_abs && aa > tol * sqrtf(fabsf(app)) * sqrtf(fabsf(aqq))) {
-            // tan of the angle, |t| <= 1; for |tau| beyond 1e18 (tau^2 would
-            // overflow) t = 1 / (2 tau) to within rounding
-            const float tau = (aqq - app) / (2.0f * apq);
-            const float at = fabsf(tau);
-            const float tn = at > 1e18f ? 0.5f / at : 1.0f / (at + sqrtf(fmaf(at, at, 1.0f)));
-            t = tau >= 0.0f ? tn : -tn;
-            c = 1.0f / sqrtf(fmaf(t, t, 1.0f));
+          const bool some = aa > floor_abs;
+          // the rotation is formed beside the test, not after it: tan of the angle,
+          // |t| <= 1; for |tau| beyond 1e18 (tau^2 would overflow) t = 1 / (2 tau) to
+          // within rounding
+          const float tau = (aqq - app) / (some ? 2.0f * apq : 1.0f);
+          const float at = fabsf(tau);
+          const float tn = at > 1e18f ? 0.5f / at : 1.0f / (at + sqrtf(fmaf(at, at, 1.0f)));
+          const float tt = tau >= 0.0f ? tn : -tn;
+          const float cc = 1.0f / sqrtf(fmaf(tt, tt, 1.0f));
+          if (some && aa > tol * sqrtf(fabsf(app)) * sqrtf(fabsf(aqq))) {
+            t = tt;
+            c = cc;
             sn = t * c;
             go = 1;
           }
         }
-        s_p[tid] = p;
-        s_q[tid] = q;
-        s_c[tid] = c;
-        s_s[tid] = sn;
-        s_t[tid] = t;
-        s_go[tid] = go;
         // the rotated pairs and the others, each in some order: every block
         // update depends only on its own entries and its two pairs, so the
         // order of the lists does not change any result
-        if (go) {
-          s_rot[atomicAdd(&s_nrot, 1)] = tid;
-          s_any = 1;
-          s_sweep_any = 1;
-        } else {
-          s_still[atomicAdd(&s_nstill, 1)] = tid;
+        const unsigned rot = __ballot_sync(0xffffffffu, go != 0),
+                       still = __ballot_sync(0xffffffffu, in && !go), below = (1u << lane) - 1u;
+        int at = 0;
+        if (lane == 0 && rot) at = atomicAdd(&s_nrot[cnt], __popc(rot));
+        if (lane == 1 && still) at = atomicAdd(&s_nstill[cnt], __popc(still));
+        const int at_rot = __shfl_sync(0xffffffffu, at, 0),
+                  at_still = __shfl_sync(0xffffffffu, at, 1);
+        if (in) {
+          s.p[tid] = p;
+          s.q[tid] = q;
+          s.c[tid] = c;
+          s.s[tid] = sn;
+          s.t[tid] = t;
+          s.go[tid] = go;
+          if (go)
+            s.rot[at_rot + __popc(rot & below)] = tid;
+          else
+            s.still[at_still + __popc(still & below)] = tid;
         }
       }
-      __syncthreads();
-      if (s_any) {
+      b_sync();
+      const int k = s_nrot[cnt], next = cnt == 2 ? 0 : cnt + 1;
+      if (tid == 0) {
+        s.k = k;
+        const int after = next == 2 ? 0 : next + 1;
+        s_nrot[after] = s_nstill[after] = 0;
+      }
+      cnt = next;
+      if (k > 0) {
+        any = true;
+        all_arrive(kReady + copy);
         // B := J^T B J over the 2 x 2 blocks (rows of pair P, columns of pair
         // Q) that a rotation touches: with Q = thread mod h fixed (its
         // columns and rotation in registers) a thread walks the rows of every
         // rotated pair, then, if Q itself is rotated, the rows of the others.
         // A warp shares P, so the pair data it reads are broadcasts.
-        const int k = s_nrot;
-        const int groups = kSyevjThreads / h;
+        const int groups = kSyevjB / h;
         const int Q = tid % h, g = tid / h;
         if (g < groups) {
-          const int b0 = s_p[Q], b1 = s_q[Q], gq = s_go[Q];
-          const float cq = s_c[Q], sq = s_s[Q];
+          const int b0 = s.p[Q], b1 = s.q[Q], gq = s.go[Q];
+          const float cq = s.c[Q], sq = s.s[Q];
           for (int i = g; i < k; i += groups) {
-            const int P = s_rot[i];
-            const int a0 = s_p[P], a1 = s_q[P];
+            const int P = s.rot[i];
+            const int a0 = s.p[P], a1 = s.q[P];
             float x00 = sB[a0 * m + b0], x01 = sB[a0 * m + b1];
             float x10 = sB[a1 * m + b0], x11 = sB[a1 * m + b1];
             if (P == Q) {  // the rotated pair's own block: exact diagonal form
-              const float tt = s_t[P];
+              const float tt = s.t[P];
               sB[a0 * m + a0] = x00 - tt * x01;
               sB[a1 * m + a1] = x11 + tt * x01;
               sB[a0 * m + a1] = 0.0f;
               sB[a1 * m + a0] = 0.0f;
               continue;
             }
-            const float cp = s_c[P], sp = s_s[P];
+            const float cp = s.c[P], sp = s.s[P];
             float y00 = cp * x00 - sp * x10, y10 = sp * x00 + cp * x10;
             float y01 = cp * x01 - sp * x11, y11 = sp * x01 + cp * x11;
             if (gq) {
@@ -428,8 +511,8 @@ __global__ void __launch_bounds__(kSyevjThreads, 1)
           }
           if (gq)
             for (int i = g; i < h - k; i += groups) {
-              const int P = s_still[i];
-              const int a0 = s_p[P], a1 = s_q[P];
+              const int P = s.still[i];
+              const int a0 = s.p[P], a1 = s.q[P];
               const float x00 = sB[a0 * m + b0], x01 = sB[a0 * m + b1];
               const float x10 = sB[a1 * m + b0], x11 = sB[a1 * m + b1];
               sB[a0 * m + b0] = cq * x00 - sq * x01;
@@ -438,41 +521,17 @@ __global__ void __launch_bounds__(kSyevjThreads, 1)
               sB[a1 * m + b1] = sq * x10 + cq * x11;
             }
         }
-        // V := V J on the rotated pairs' columns (global memory, L2-resident):
-        // each thread loads a batch of its items before it stores any, so the
-        // loads' latencies overlap
-        for (int base = tid; base < k * n; base += kSyevjThreads * kVBatch) {
-          float vp[kVBatch], vq[kVBatch];
-          int ip[kVBatch], iq[kVBatch], pr[kVBatch];
-#pragma unroll
-          for (int u = 0; u < kVBatch; ++u) {
-            const int e = base + kSyevjThreads * u;
-            pr[u] = -1;
-            if (e < k * n) {
-              const int P = s_rot[e / n], row = e % n;
-              pr[u] = P;
-              ip[u] = row + n * s_p[P];
-              iq[u] = row + n * s_q[P];
-              vp[u] = V[ip[u]];
-              vq[u] = V[iq[u]];
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < kVBatch; ++u) {
-            if (pr[u] < 0) continue;
-            const float c = s_c[pr[u]], sn = s_s[pr[u]];
-            V[ip[u]] = c * vp[u] - sn * vq[u];
-            V[iq[u]] = sn * vp[u] + c * vq[u];
-          }
-        }
+        copy ^= 1;
+        if (++used > 1) all_sync(kDone + copy);  // V is done with the copy's last round
+        else b_sync();
       }
-      __syncthreads();
     }
     sweeps = sweep;
-    converged = (s_sweep_any == 0);
-    __syncthreads();
+    converged = !any;
   }
-  for (int i = tid; i < n; i += blockDim.x) lam[i] = sB[i * m + i];
+  if (tid == 0) s_pairs[copy].k = -1;
+  all_arrive(kReady + copy);
+  for (int i = tid; i < n; i += kSyevjB) lam[i] = sB[i * m + i];
   if (tid == 0) *sweeps_out = converged ? sweeps : -max_sweeps;
 }
 
