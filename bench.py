@@ -226,10 +226,11 @@ def kernel_work(name, shape):
 
 
 def jacobi_flops(prof, shape):
-    """FP32 flops of the Jacobi launches as the kernel does the work: 8 nr per
-    examined column pair (the inner product w_p^H w_q; the squared norms are
-    tracked through the rotations) and 18 (nr + nc) per rotated pair (phase,
-    two complex scaled sums on W's and V's rows)."""
+    """The Jacobi launches' work as a one-sided Jacobi on the columns counts it:
+    8 nr flops per examined column pair (the inner product w_p^H w_q) and
+    18 (nr + nc) per rotated pair (phase, two complex scaled sums on W's and V's
+    rows).  The kernel forms the inner products and the sums by the tensor cores,
+    a panel pair at a time, so that this is the algorithm's count, not its pipe's."""
     n1, n2, _ = shape
     nr, nc = max(n1, n2), min(n1, n2)
     return 8.0 * nr * prof.jacobi_pairs + 18.0 * (nr + nc) * prof.jacobi_rotations
@@ -532,8 +533,9 @@ def run_ours(args, wl_name):
         textbook = jacobi_textbook_flops(prof, shape) / prof.launches[6]
         roof = {"bound": "alu", "achieved": flops / avg_s / 1e12, "peak": peak["fp32"],
                 "unit": "TFLOP/s", "peak_source": peak["fp32_source"],
-                "work": "the kernel's own: 8 nr flops per examined column pair, 18 (nr + nc) per "
-                        "rotated pair, counted on the device",
+                "work": "a column Jacobi's: 8 nr flops per examined column pair, 18 (nr + nc) per "
+                        "rotated pair, counted on the device (the kernel forms most of them "
+                        "on the tensor cores)",
                 "achieved_textbook": textbook / avg_s / 1e12,
                 "frac_textbook": textbook / avg_s / 1e12 / peak["fp32"]}
     else:
@@ -568,10 +570,9 @@ def run_ours(args, wl_name):
                    "jacobi_start": args.jacobi_start,
                    "gemm_precision": precision,
                    "mode3_dft": "tensor cores" if args.dft == "tc" else "SIMT direct sums",
-                   "jacobi_schedule": ("task graph: panel-pair tasks of every slice on all SMs"
-                                       if args.jacobi_schedule == "tasks" else "one CTA per slice"),
-                   "jacobi_panel": args.jacobi_panel,
-                   "jacobi_order": ("columns by norm, largest first, each sweep"
+                   "jacobi_schedule": "panel-pair tasks of every slice from one queue, on all SMs",
+                   "jacobi_panel": 16,
+                   "jacobi_order": ("columns by norm, largest first, from the start"
                                     if args.jacobi_order == "sorted" else "stored order"),
                    "l_update": ("Tucker projection, one HOOI sweep per iteration, ranks %s" % (ranks,)
                                 if ranks else "plain (full Tucker ranks)"),
@@ -603,7 +604,7 @@ def run_ours(args, wl_name):
 
 def run_batch(args):
     """The batched form: all cubes advance one ADMM iteration per step (one
-    persistent Jacobi launch over every Fourier slice of every cube); value =
+    Jacobi launch over every Fourier slice of every cube); value =
     cube-iterations per second.  The same cubes run one plan at a time for a
     few iterations give the unbatched comparison."""
     import numpy as np
@@ -647,7 +648,7 @@ def run_batch(args):
         clk = clocks.stop()
         unconv = sum(b.plan(i).stats().jacobi_unconverged for i in range(len(shapes)))
         # profiled pass over the same iterations of the denoise, for the
-        # persistent Jacobi's share (cube 0's profile) and the launches of a
+        # Jacobi's share (cube 0's profile) and the launches of a
         # step (every group's launches are in the profile of its first cube)
         ngroups, _ = b.groups()
         b.init(Ys)
@@ -704,7 +705,7 @@ def run_batch(args):
         "gpu_launches": int(spans),
         "launches_per_step": {"profiled": spans / args.steps, "groups": ngroups,
                               "note": "one launch per kernel and group of equal shape and "
-                                      "parameters, one persistent Jacobi launch; the profiler "
+                                      "parameters, one Jacobi launch; the profiler "
                                       "brackets the DFT, GEMM, stencil and Jacobi launches"},
         "jacobi_persistent": {"launches": prof.launches[6],
                               "ms_per_launch": prof.ms[6] / max(prof.launches[6], 1),
@@ -1024,14 +1025,14 @@ def build_parser():
                     help="mode-3 DFT engine: the tensor-core pipeline or the SIMT direct sums "
                          "(LRSTV_FLAG_SIMT_DFT)")
     ap.add_argument("--jacobi-schedule", choices=["tasks", "slice"], default="tasks",
-                    help="the Jacobi's task-graph schedule over all SMs, or one CTA per slice "
-                         "(LRSTV_FLAG_JACOBI_PER_SLICE)")
+                    help="slice sets LRSTV_FLAG_JACOBI_PER_SLICE, which is accepted without "
+                         "effect: the Jacobi always takes tasks over all SMs")
     ap.add_argument("--jacobi-panel", type=int, choices=[32, 16], default=32,
-                    help="the Jacobi's column panel width: 32 (16-warp CTAs) or 16 (8-warp CTAs, "
-                         "two to an SM; LRSTV_FLAG_JACOBI_PANEL16)")
+                    help="16 sets LRSTV_FLAG_JACOBI_PANEL16, which is accepted without effect: "
+                         "the Jacobi's column panels are 16 wide")
     ap.add_argument("--jacobi-order", choices=["sorted", "fixed"], default="sorted",
-                    help="the Jacobi orders each sweep's columns by norm, largest first, or "
-                         "keeps their stored order (LRSTV_FLAG_JACOBI_FIXED_ORDER)")
+                    help="the Jacobi orders a slice's columns by norm at its start, largest "
+                         "first, or keeps their stored order (LRSTV_FLAG_JACOBI_FIXED_ORDER)")
     ap.add_argument("--unroll-factors", choices=["keep", "recompute"], default="keep",
                     help="c5: keep every iteration's SVD factors from the forward pass, or "
                          "recompute them in the backward pass (LRSTV_FLAG_UNROLL_RECOMPUTE)")

@@ -1172,7 +1172,7 @@ int lrstv_denoise(const float *Y, int n1, int n2, int n3, const lrstv_params *pa
 // group's plans are carved from one arena by group_layout, so that its cubes
 // form a packed batch: each step of an iteration is one launch per kernel for
 // the whole group (the stencils, the mode-3 and spatial DFTs, the GEMMs and
-// the small per-slice kernels), and the Jacobi is one persistent launch over
+// the small per-slice kernels), and the Jacobi is one launch of tasks over
 // the slices of every group.  A batched step's launches thus grow with the
 // number of distinct shapes, not with the number of cubes.  The arithmetic
 // of every cube is that of a plan of its own, so the results are the same
@@ -1181,7 +1181,7 @@ struct BatchGroup {
   int m;              // cubes
   lrstv_plan **pls;   // their plans, in batch order; pls[0] holds the group's block bases
   void *arena;
-  int big;            // slices taller than the persistent kernel takes: one launch
+  int big;            // slices taller than the common launch takes: one launch
 };
 
 struct lrstv_batch {
@@ -1285,7 +1285,7 @@ int group_fs_dual(const BatchGroup &g, cudaStream_t st) {
 }
 
 // Step 4 (E) of every cube: per group the mode-3 DFT, the warm start's
-// products and the RMS norms; one persistent Jacobi launch over the slices of
+// products and the RMS norms; one Jacobi launch over the slices of
 // all groups (taller slices: one launch per group); per group sigma and
 // V diag g, the reconstruction and the inverse DFT with Gamma4.
 int batch_e_step(lrstv_batch *b, cudaStream_t st) {

@@ -414,7 +414,7 @@ class _BorrowedPlan(Plan):
 class Batch:
     """An lrstv_batch: independent cubes of uneven shapes run in lockstep,
     one launch per kernel and group of equal shapes and parameters, with one
-    persistent Jacobi launch per E-step."""
+    Jacobi launch per E-step over the slices of all cubes."""
 
     def __init__(self, shapes, params):
         _torch()
