@@ -1606,7 +1606,8 @@ cudaError_t blk_launch(Run a, cudaStream_t st) {
   long long grid = (long long)per_sm * nsm;
   if (grid > 2ll * a.nslices * width) grid = 2ll * a.nslices * width;
   // slices in flight: their operands within about 96 MB of the 129 MB L2, and
-  // enough of them to give every worker two tasks
+  // enough of them to give every worker two tasks (1.5 tasks: 200 x 200 x 80, 50
+  // iterations, 115 -> 134 ms; three, four or all slices: within 1%)
   const long long bytes = (long long)op_bytes(a.nr, a.nc);
   long long live = (96ll << 20) / bytes;
   const long long least = (2 * grid + width - 1) / width;
