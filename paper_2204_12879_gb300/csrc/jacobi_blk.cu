@@ -363,9 +363,10 @@ __device__ float norms_and_sum(int nr, int nc, const float2 *W, float *key, floa
   return sum;
 }
 
-// The power of two that scales W for the FP16 split: ||W||_F s in [2^14, 2^15).
+// The power of two that scales W for the FP16 split: ||W||_F s in [2^14, 2^15),
+// for every finite ||W||_F^2 (slice_start lets no other slice run).
 __device__ __forceinline__ float w_scale(float fro2) {
-  if (!(fro2 > 0.0f) || !(fro2 < 3e38f)) return 1.0f;
+  if (!(fro2 > 0.0f) || !(fro2 <= FLT_MAX)) return 1.0f;
   int e = ilogbf(sqrtf(fro2));
   e = e < -100 ? -100 : (e > 100 ? 100 : e);
   return ldexpf(1.0f, 14 - e);
