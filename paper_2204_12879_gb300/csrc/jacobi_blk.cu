@@ -43,9 +43,11 @@
 // Schedules.  Tasks: every CTA takes tasks of any slice from a queue in global
 // memory; a scheduler warp claims tasks, counts them off and queues the next
 // round while the eight worker warps run.  Per slice: one CTA runs a slice's
-// tasks one after another on W and V in place (for calls that have no
-// scratch).  The pairs of a round touch disjoint columns and both schedules do
-// the same arithmetic, so a slice's result is the same on either.
+// tasks one after another on W and V in place (for calls that have no scratch,
+// slices above 256 rows; smaller ones are faster in FP32, svt.cu).  The pairs of
+// a round touch disjoint columns and both schedules do the same arithmetic, so a
+// slice's result is the same on either up to rounding: a value kept in FP32
+// between two tasks and split again may get other halves of the same sum.
 //
 // What bounds it: the latency of a task's chain (16 rotation rounds of two
 // barriers each, two loads, three MMA waits); 72 registers and one region of
@@ -1451,7 +1453,9 @@ __global__ void __launch_bounds__(kT, 3) k_jacobi_tasks(Run a) {
 }
 
 // The per-slice schedule: CTA b runs the tasks of slice b one after another on
-// W and V in place.
+// W and V in place.  Gathering and splitting a task's columns every time makes it
+// slower than the FP32 kernel where that holds a panel in registers (up to 256
+// rows, see launch_jacobi).
 __global__ void __launch_bounds__(kT, 2) k_jacobi_slices(Run a) {
   extern __shared__ __align__(128) char smem[];
   __shared__ __align__(8) uint64_t s_bar[7];

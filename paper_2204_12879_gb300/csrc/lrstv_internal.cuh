@@ -164,8 +164,8 @@ struct JacOpt {
   int group = 1;
   float negl_rel = -1.0f;
   // scratch of jacobi_task_ints(nslices, nc, nslices jacobi_op_bytes(nr, nc))
-  // ints: with it, every SM takes tasks of any slice from a queue; without it,
-  // one CTA runs a slice
+  // ints: with it, every SM takes tasks of any slice from a queue (blocked kernel);
+  // without it, one CTA runs a slice (up to 256 rows on the FP32 kernel)
   int *sched = nullptr;
   // nslices flags of launch_gram_check (may be null): a slice whose flag is
   // set ends after one sweep without running it (that sweep would rotate
@@ -195,9 +195,10 @@ cudaError_t launch_gram_check(const Dims &d, int nslices, const float2 *W, float
 // take op_total bytes (256-byte aligned).
 size_t jacobi_op_bytes(int nr, int nc);
 size_t jacobi_task_ints(int nslices, int nc, size_t op_total);
-// The blocked kernel (jacobi_blk.cu), or, when negl_rel is given (the Tucker
-// eigen-solves, whose null-space columns the blocked kernel's FP16 halves
-// would not resolve), the per-slice FP32 kernels (svt.cu).
+// The blocked kernel (jacobi_blk.cu), or the per-slice FP32 kernels (svt.cu): for
+// slices of up to 256 rows without a queue's scratch, and when negl_rel is given
+// (the Tucker eigen-solves, whose null-space columns the blocked kernel's FP16
+// halves would not resolve).
 cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, float t,
                           int max_sweeps, int *sweeps, unsigned long long *work,
                           cudaStream_t st, const JacOpt &opt = JacOpt());

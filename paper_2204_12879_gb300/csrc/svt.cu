@@ -1,7 +1,8 @@
 // svt.cu -- the small kernels around the t-SVT's Jacobi (arXiv 2204.12879, eq.
 // E_solution; the slice-wise form follows Theorem 4.2's t-SVD): the RMS norms,
-// the Gram pre-check, sigma and V diag g; and the FP32 one-sided Jacobi that the
-// Tucker L-update's eigen-solves take.
+// the Gram pre-check, sigma and V diag g; and the FP32 one-sided Jacobi of the
+// calls without a task queue's scratch (slices of up to 256 rows, one CTA each) and
+// of the Tucker L-update's eigen-solves.
 //
 // The FP32 Jacobi orthogonalises a working matrix W (nr x nc complex, nr >= nc)
 // by one-sided (Hestenes) rotations of column pairs (p, q) until
@@ -15,7 +16,7 @@
 //    instructions (__ffma2_rn) on a split row-pair layout;
 //  - k_jacobi (any nr up to 512): round-robin over all columns in global
 //    memory (L2-resident), one pair per warp.
-// The Fourier slices' SVDs are jacobi_blk.cu's.
+// The other Fourier slices' SVDs are jacobi_blk.cu's.
 #include <float.h>
 
 #include "jacobi_common.cuh"
@@ -650,7 +651,7 @@ template <int KP, int PW>
 __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float2 *V, float t,
                                                 int max_sweeps, float tol, float negl_rel,
                                                 int *sweeps_slot, unsigned long long *work,
-                                                float4 *smem, int warm) {
+                                                float4 *smem, const JacOpt &o, int slice) {
   constexpr int LD2 = PkShape<KP>::LD2;
   float4 *sW = smem;              // panel a (own pairs), then panel b: W
   float4 *sVa = sW + PW * LD2;    // panel a: V
@@ -667,17 +668,33 @@ __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float
   __shared__ int s_perm[kSortCols];
   __shared__ float s_key[kSortCols];
 
-  const float fro2 = pk_setup<false>(nr, nc, W, V, warm, s_red);
+  const float fro2 = pk_setup<false>(nr, nc, W, V, o.warm, s_red);
   const float negl = negl_rel * fro2;
   const int npan = (nc + PW - 1) / PW;
   unsigned n_pairs = 0, n_rot = 0;  // lane 0 (own pairs) and ul 0 (cross pairs) count
   int sweeps = (nc < 2) ? 1 : 0;
   bool converged = (nc < 2);
+  // every singular value is at most ||W||_F: at or below the threshold the SVT
+  // is zero whatever the sweeps would find, so none is run
+  if (o.t_svt >= 0.0f && fro2 <= o.t_svt * o.t_svt) {
+    sweeps = 0;
+    converged = true;
+  }
+  // the Gram check showed that a sweep would rotate no pair
+  if (!converged && o.conv && o.conv[slice]) {
+    sweeps = 1;
+    converged = true;
+  }
+  tol = pk_tolerance(tol, fro2, nc, o.t_svt, o.ms2 ? o.ms2[slice / o.group] : -1.0f);
   float4 aW[KP], aV[KP];
-  if (!converged) {  // the first sweep's order: by the columns' norms
-    col_norms(nr, nc, W, s_key);
-    __syncthreads();
-    order_columns(nc, s_key, s_perm);
+  if (!converged) {  // the first sweep's order: by the columns' norms, or as stored
+    if (o.sort) {
+      col_norms(nr, nc, W, s_key);
+      __syncthreads();
+      order_columns(nc, s_key, s_perm);
+    } else {
+      for (int c = tid; c < nc; c += blockDim.x) s_perm[c] = c;
+    }
   }
   for (int sweep = 1; sweep <= max_sweeps && !converged; ++sweep) {
     if (tid == 0) s_rot = 0;
@@ -712,7 +729,7 @@ __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float
     sweeps = sweep;
     converged = (s_rot == 0);
     // the next sweep's order, from the norms this one left
-    if (!converged) order_columns(nc, s_key, s_perm);
+    if (o.sort && !converged) order_columns(nc, s_key, s_perm);
     __syncthreads();
   }
   pk_epilogue<false>(nr, nc, W, V, t);
@@ -733,7 +750,7 @@ __global__ void __launch_bounds__(PW * 16, (KP <= 2 || PW == 16) ? 2 : 1)
   extern __shared__ float4 smem_f4[];
   const int s = blockIdx.x;
   jacobi_pk_slice<KP, PW>(nr, nc, W_all + (size_t)s * wstride, V_all + (size_t)s * vstride, t,
-                          max_sweeps, tol, negl_rel, sweeps_out + s, work, smem_f4, o.warm);
+                          max_sweeps, tol, negl_rel, sweeps_out + s, work, smem_f4, o, s);
 }
 
 template <int KP>
@@ -925,16 +942,23 @@ cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, floa
                           cudaStream_t st, const JacOpt &o) {
   const int nr = d.nr, nc = d.nc;
   if (nslices <= 0) return cudaSuccess;
-  if (o.negl_rel < 0.0f)
+  // Without a queue's scratch one CTA runs a slice: up to 256 rows the FP32 kernel,
+  // which keeps a panel in registers while the others stream past (200 x 200 x 80:
+  // 10.5 ms a t-SVT against 23.3 with the blocked kernel's tasks one after another,
+  // 64 x 64 x 31: 0.68 against 0.82, 32 x 32 x 16: 0.23 against 0.21); above, the
+  // blocked one (280 x 300 x 31: 53 ms against k_jacobi's 84).
+  const bool eig = o.negl_rel >= 0.0f;
+  if (!eig && (o.sched || nr > 256))
     return launch_jacobi_blk(d, nslices, W, V, t, max_sweeps, sweeps, work, st, o);
   const int np = nc + (nc & 1);
   const int R = (nr + 31) / 32;
   int pairs = np / 2 < 1 ? 1 : np / 2;
   const int maxw = R <= 8 ? 32 : 16;
   const int nw = pairs < maxw ? pairs : maxw;
-  const float tol = jacobi_tol0(nr), negl = o.negl_rel;
+  const float eps = FLT_EPSILON * 0.5f;
+  const float tol = jacobi_tol0(nr), negl = eig ? o.negl_rel : ((float)nr * eps) * ((float)nr * eps);
   const size_t ws = d.P, vs = (size_t)nc * nc;
-  if (nr <= 256 && nc >= 2) {
+  if (nr <= 256) {
     const int KP = R;
 #define LRSTV_PK(K) \
   return launch_pk<K>(nslices, nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o, st)
