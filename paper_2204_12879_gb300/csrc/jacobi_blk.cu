@@ -1103,9 +1103,11 @@ __global__ void __launch_bounds__(1024) k_blk_setup(Run a) {
 }
 
 // Closing launch of the task schedule: a slice's operands back to W and V, and
-// g_i = max(1 - t / sigma_i, 0) applied to V (t >= 0).  One CTA a panel.
-__global__ void __launch_bounds__(256) k_blk_close(Run a) {
-  __shared__ float s_n2[8][kB];
+// g_i = max(1 - t / sigma_i, 0) applied to V (t >= 0), summed in the order of the
+// other kernels' epilogues.  A slice whose first sweep rotated nothing keeps the W
+// and V it came with, not their 22-bit halves: as if the sweep had not run.  One
+// CTA a panel, a warp a column.
+__global__ void __launch_bounds__(32 * kB) k_blk_close(Run a) {
   __shared__ float s_g[kB];
   __shared__ int s_col[kB];
   const int s = blockIdx.x, p = blockIdx.y;
@@ -1113,54 +1115,60 @@ __global__ void __launch_bounds__(256) k_blk_close(Run a) {
   if (!q.packed[s]) return;
   const Slice x = slice_of(a, s);
   const int npan = panels_of(x.nc);
-  if (p >= npan) return;
+  const bool still = *x.sweeps == 1;
+  if (p >= npan || (still && x.warm && x.t < 0.0f)) return;
   if (threadIdx.x < kB) {
     const int at = p * kB + threadIdx.x;
     s_col[threadIdx.x] = at < x.nc ? q.perm[(size_t)a.cols * s + at] : -1;
+    s_g[threadIdx.x] = 1.0f;
   }
   __syncthreads();
   const int np = players_of(npan), rw = rows16(x.nr), rv = rows16(x.nc);
   auto unpack = [&](const char *src, int rows, int n, float2 *M, float inv, bool isv) {
-    float n2[kB] = {};
-    for (int r = threadIdx.x; r < n; r += 256) {
+    for (int u = threadIdx.x; u < 2 * n; u += 32 * kB) {
+      const int g = u >= n, r = u - g * n;
+      const char *b = src + ((size_t)g * rows + r) * 16;
+      const size_t st = (size_t)rows * 32;
+      float re[8] = {}, im[8] = {};
+      join8(*(const uint4 *)b, *(const uint4 *)(b + st), re);
+      join8(*(const uint4 *)(b + 2 * st), *(const uint4 *)(b + 3 * st), im);
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const char *b = src + ((size_t)g * rows + r) * 16;
-        const size_t st = (size_t)rows * 32;
-        float re[8] = {}, im[8] = {};
-        join8(*(const uint4 *)b, *(const uint4 *)(b + st), re);
-        join8(*(const uint4 *)(b + 2 * st), *(const uint4 *)(b + 3 * st), im);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int c = s_col[8 * g + j];
-          float2 v = make_float2(re[j] * inv, im[j] * inv);
-          if (isv && x.t >= 0.0f) {
-            v.x *= s_g[8 * g + j];
-            v.y *= s_g[8 * g + j];
-          }
-          n2[8 * g + j] = fmaf(v.x, v.x, fmaf(v.y, v.y, n2[8 * g + j]));
-          if (c >= 0) M[(size_t)n * c + r] = v;
+      for (int j = 0; j < 8; ++j) {
+        const int c = s_col[8 * g + j];
+        float2 v = make_float2(re[j] * inv, im[j] * inv);
+        if (isv) {
+          v.x *= s_g[8 * g + j];
+          v.y *= s_g[8 * g + j];
         }
+        if (c >= 0) M[(size_t)n * c + r] = v;
       }
     }
-    if (isv || x.t < 0.0f) return;
-#pragma unroll
-    for (int j = 0; j < kB; ++j) {
-      const float v = warp_sum(n2[j]);
-      if ((threadIdx.x & 31) == 0) s_n2[threadIdx.x >> 5][j] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kB) {
-      float v = 0.0f;
-      for (int w = 0; w < 8; ++w) v += s_n2[w][threadIdx.x];
-      const double sigma = sqrt((double)v);
-      s_g[threadIdx.x] =
-          sigma > (double)x.t ? (float)(1.0 - (double)x.t / sigma) : 0.0f;
-    }
-    __syncthreads();
   };
-  unpack(x.op + (size_t)p * rw * 128, rw, x.nr, x.W, q.lim[s].w, false);
-  unpack(x.op + ((size_t)np * rw + (size_t)p * rv) * 128, rv, x.nc, x.V, 1.0f / kScaleV, true);
+  if (!still) unpack(x.op + (size_t)p * rw * 128, rw, x.nr, x.W, q.lim[s].w, false);
+  if (x.t >= 0.0f) {
+    __syncthreads();
+    const int j = threadIdx.x >> 5;
+    if (s_col[j] >= 0) {
+      const float n2 = column_norm2<false>(x.nr, x.W + (size_t)x.nr * s_col[j]);
+      if ((threadIdx.x & 31) == 0) s_g[j] = n2;
+    }
+    __syncthreads();
+    // FP64 by sixteen threads: with every lane of the warps the kernel took 16.4 us at
+    // 75 x 91 x 220, so 10.8
+    if (threadIdx.x < kB && s_col[threadIdx.x] >= 0) s_g[threadIdx.x] = gain(s_g[threadIdx.x], x.t);
+    __syncthreads();
+  }
+  if (!still) {
+    unpack(x.op + ((size_t)np * rw + (size_t)p * rv) * 128, rv, x.nc, x.V, 1.0f / kScaleV, true);
+    return;
+  }
+  for (int e = threadIdx.x; e < kB * x.nc; e += 32 * kB) {
+    const int j = e / x.nc, r = e - j * x.nc, c = s_col[j];
+    if (c < 0) continue;
+    float2 *v = x.V + (size_t)x.nc * c + r;
+    const float2 u = x.warm ? *v : make_float2(c == r ? 1.0f : 0.0f, 0.0f);
+    *v = make_float2(u.x * s_g[j], u.y * s_g[j]);
+  }
 }
 
 // TMEM and barriers of a CTA (every thread); `tasks`: those of the task schedule too
@@ -1627,7 +1635,7 @@ cudaError_t blk_launch(Run a, cudaStream_t st) {
   else
     k_jacobi_tasks<false><<<(unsigned)grid, kT, ops + kScratch<false>, st>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_blk_close<<<dim3(a.nslices, panels_of(a.cols)), 256, 0, st>>>(a);
+  k_blk_close<<<dim3(a.nslices, panels_of(a.cols)), 32 * kB, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -99,22 +99,31 @@ __device__ __forceinline__ float pk_tolerance(float tol, float fro2, int nc, flo
   return tol;
 }
 
-// g_i = max(1 - t / sigma_i, 0) applied to V's columns (t < 0: V unscaled),
-// sigma_i = |w_i|; the sigma-vs-t decision is taken in FP64.
+// |w|^2 of a column by one warp, in the order of every epilogue
+template <bool CG>
+__device__ __forceinline__ float column_norm2(int nr, const float2 *w) {
+  float n2 = 0.f;
+  for (int row = threadIdx.x & 31; row < nr; row += 32) {
+    const float2 x = ldw<CG>(w + row);
+    n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, n2));
+  }
+  return warp_sum(n2);
+}
+
+// g = max(1 - t / sigma, 0) of a column of squared norm n2; the sigma-vs-t decision
+// is taken in FP64.
+__device__ __forceinline__ float gain(float n2, float t) {
+  const double sigma = sqrt((double)n2);
+  return sigma > (double)t ? (float)(1.0 - (double)t / sigma) : 0.0f;
+}
+
+// g_i = max(1 - t / sigma_i, 0) applied to V's columns (t < 0: V unscaled).
 template <bool CG>
 __device__ __forceinline__ void pk_epilogue(int nr, int nc, const float2 *W, float2 *V, float t) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (t < 0.0f) return;
   for (int i = warp; i < nc; i += (int)(blockDim.x >> 5)) {
-    const float2 *wi = W + (size_t)nr * i;
-    float n2 = 0.f;
-    for (int row = lane; row < nr; row += 32) {
-      const float2 x = ldw<CG>(wi + row);
-      n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, n2));
-    }
-    n2 = warp_sum(n2);
-    const double sigma = sqrt((double)n2);
-    const float g = sigma > (double)t ? (float)(1.0 - (double)t / sigma) : 0.0f;
+    const float g = gain(column_norm2<CG>(nr, W + (size_t)nr * i), t);
     float2 *vi = V + (size_t)nc * i;
     for (int row = lane; row < nc; row += 32) {
       const float2 v = ldw<CG>(vi + row);

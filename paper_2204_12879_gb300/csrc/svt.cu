@@ -826,12 +826,14 @@ __global__ void k_gram_gate(const int *__restrict__ sweeps, int n, int *__restri
 
 // conv[s] for the Gram matrix G_s (nc x nc, column-major) of a candidate slice:
 // 1 when every pair p < q passes |G_pq| <= (tol (1 - 1e-3) - kappa) sqrt(G_pp G_qq).
-// The sweep rotates a pair when |g|^2 > tol^2 |w_p|^2 |w_q|^2 with g its own FP32
-// inner product; G_pq carries at most about (nr eps + 2^-20) |w_p| |w_q| of
-// rounding (3xTF32 products, FP32 sums) and g about nr eps |w_p| |w_q|, so
-// kappa = 4 nr eps + 4e-6 keeps every passing pair below the sweep's test, and
-// the (1 - 1e-3) covers the sweep's own squared norms and this test's FP32
-// squares.  tol: the Jacobi's threshold-aware tolerance (pk_tolerance with the
+// The sweep rotates a pair when |g|^2 > tol^2 |w_p|^2 |w_q|^2 with g the inner
+// product of its own Gram.  G_pq carries at most about (nr eps + 2^-20) |w_p| |w_q|
+// of rounding (3xTF32 products, FP32 sums); g carries the 22-bit halves' 2^-22
+// and the tensor core's truncation, one ulp (2 eps) of at most |w_p| |w_q| for each
+// 16 rows and each of the four split products, of which hi*hi alone is full-size:
+// nr eps / 8 and a little.  kappa = 4 nr eps + 4e-6 keeps every passing pair below
+// the sweep's test, and the (1 - 1e-3) covers the sweep's own squared norms and
+// this test's FP32 squares.  tol: the Jacobi's threshold-aware tolerance (pk_tolerance with the
 // tensor's ms2).  One CTA a slice.
 __global__ void __launch_bounds__(256)
     k_gram_check(const float2 *__restrict__ G, int nr, int nc, const int *__restrict__ cand,
