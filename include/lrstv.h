@@ -342,7 +342,7 @@ int lrstv_denoise(const float *Y, int n1, int n2, int n3, const lrstv_params *pa
  *          may differ.  Parameters are fixed when the batch is created.
  * The batch owns one plan per cube (lrstv_batch_plan lends it for stats and
  * state export; do not destroy it or change its parameters), one allocation
- * per group and one small allocation for the work list.  Slices taller than
+ * per group and one small allocation for the work list and the task queue.  Slices taller than
  * 256 rows (max(n1, n2)) take a separate Jacobi launch per cube.  The
  * Jacobi launch is recorded in cube 0's profile (lrstv_profile_*), a
  * group's other launches in the profile of its first cube.  A cube whose plan

@@ -1189,10 +1189,10 @@ struct lrstv_batch {
   lrstv_plan **plans;
   int ngroups;
   BatchGroup *groups;
-  void *arena;           // the slice work list and its counter
+  void *arena;           // the slice work list and the task queue
   SliceTask *d_tasks;
   int ntasks;
-  int *d_sched;          // the task queue's scratch
+  int *d_sched;          // the task queue's scratch (the operands are the plans')
   int max_nr, max_nc;    // the largest slice sides in the work list
   cudaStream_t cap_stream;
   cudaGraphExec_t gexec;
@@ -1485,7 +1485,6 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
     return rc;
   }
   int ntasks = 0, maxnr = 1, maxnc = 1;
-  size_t op = 0;
   for (int i = 0; i < ncubes; ++i) {
     const Dims &d = b->plans[i]->d;
     if (d.nr <= kBatchMaxNr) {
@@ -1517,14 +1516,15 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
         // the Gram check runs with the warm start on the tensor-core engine
         h[k].conv = ((pl->prm.flags & LRSTV_FLAG_WARM_START) && plan_gemm(pl).tc)
                         ? pl->gconv + s : nullptr;
-        h[k].op = op;
-        op += jacobi_op_bytes(d.nr, d.nc);
+        // its plan's, which no launch of the plan's own uses meanwhile
+        h[k].op = (char *)(pl->jsched + jacobi_task_ints(3 * d.h, d.nc, 0)) +
+                  (size_t)s * jacobi_op_bytes(d.nr, d.nc);
         ++k;
       }
     }
     qsort(h, (size_t)ntasks, sizeof(SliceTask), task_cmp);
     const size_t tbytes = align_up(sizeof(SliceTask) * (size_t)ntasks);
-    if (cudaMalloc(&b->arena, tbytes + sizeof(int) * jacobi_task_ints(ntasks, maxnc, op)) !=
+    if (cudaMalloc(&b->arena, tbytes + sizeof(int) * jacobi_task_ints(ntasks, maxnc, 0)) !=
         cudaSuccess) {
       cudaGetLastError();
       delete[] h;

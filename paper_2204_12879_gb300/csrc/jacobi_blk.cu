@@ -281,7 +281,7 @@ struct Run {
   double mu;
   int keep;
   int *sched;
-  char *op;                 // the operands (one shape: slice s at op + s op_bytes)
+  char *op;                 // one shape: the operands, slice s at op + s op_bytes
   int cap, cols;
   int live_max;             // slices in flight at most (task schedule)
   int rows;                 // rows of the tallest slice, rounded up to 16
@@ -306,7 +306,7 @@ __device__ __forceinline__ Slice slice_of(const Run &a, int s) {
     x.nc = tk.nc;
     x.W = tk.W;
     x.V = tk.V;
-    x.op = a.op + tk.op;
+    x.op = tk.op;
     x.skip_t = (float)((double)tk.alpha / a.mu);
     x.t = a.keep ? -1.0f : x.skip_t;
     x.tol0 = 8.0f * sqrtf((float)tk.nr) * eps;
@@ -1371,7 +1371,7 @@ __global__ void __launch_bounds__(kT, 3) k_jacobi_tasks(Run a) {
           r = (task / kMaxTasks) % kMaxRounds;
           nr = a.list ? a.list[s].nr : a.nr;
           nc = a.list ? a.list[s].nc : a.nc;
-          char *op = a.op + (a.list ? a.list[s].op : (size_t)s * op_bytes(nr, nc));
+          char *op = a.list ? a.list[s].op : a.op + (size_t)s * op_bytes(nr, nc);
           npan = panels_of(nc);
           const int rw = rows16(nr), rv = rows16(nc);
           round_pair(npan, r, task % kMaxTasks, pa, pb);

@@ -192,7 +192,8 @@ cudaError_t launch_gram_check(const Dims &d, int nslices, const float2 *W, float
                               const float *ms2, int group, int *gemm_err, cudaStream_t st);
 // Scratch of the blocked kernel's task schedule: bytes of one slice's operands,
 // and ints for nslices working matrices of up to nc columns whose operands
-// take op_total bytes (256-byte aligned).
+// take op_total bytes (256-byte aligned; they follow jacobi_task_ints(nslices,
+// nc, 0) ints).
 size_t jacobi_op_bytes(int nr, int nc);
 size_t jacobi_task_ints(int nslices, int nc, size_t op_total);
 // The blocked kernel (jacobi_blk.cu), or the per-slice FP32 kernels (svt.cu): for
@@ -229,15 +230,15 @@ struct SliceTask {
   int nr, nc;
   const float *ms2;  // the slice's group value of launch_group_ms2 (may be null)
   const int *conv;   // the slice's launch_gram_check flag (may be null)
-  size_t op;         // the slice's operands: their offset in the scratch's operand part
+  char *op;          // the slice's operands (jacobi_op_bytes, 256-byte aligned)
 };
 // Largest slice height of a batch's common launch (taller slices would leave
 // one CTA to an SM for all of them).
 constexpr int kBatchMaxNr = 256;
 // The blocked Jacobi over a list of slices of any shapes up to max_nr x max_nc.
 // warm: as launch_jacobi; keep: V left unscaled (threshold taken as negative);
-// sort: as JacOpt::sort; sched: jacobi_task_ints(nslices, max_nc, the slices'
-// jacobi_op_bytes together) ints.
+// sort: as JacOpt::sort; sched: jacobi_task_ints(nslices, max_nc, 0) ints (the
+// operands are the list's).
 cudaError_t launch_jacobi_list(const SliceTask *list, int nslices, int max_nr, int max_nc,
                                double mu, int max_sweeps, unsigned long long *work,
                                cudaStream_t st, int warm, int keep, int sort, int *sched);
