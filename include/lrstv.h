@@ -385,9 +385,10 @@ int lrstv_zsolve_workspace_size(int n1, int n2, int n3, size_t *bytes);
 int lrstv_tsvt_workspace_size(int n1, int n2, int n3, size_t *bytes);
 /* Z = ifftn(fftn(T) / (mu (1 + P_z))), P_z = sum_n w_n^2 |fftn(D_n)|^2
  * (eq. Z_solution).  The products run on the tensor cores, FP32-accurate (3xTF32,
- * small products first): about 4e-7 of ||Z|| off at 145 x 145 x 220 (a cube whose
- * values are all below about 1e-33 loses digits: the split's low halves leave
- * FP32's normal range).  ERR_ARG if the workspace is too small. */
+ * small products first): about 4e-7 of ||Z|| off at 145 x 145 x 220, at any
+ * magnitude of T that FP32 sums allow (what lies below about 1e-28, where the
+ * split's low halves would leave FP32's normal range, takes FP32 FMAs, ten
+ * times slower).  ERR_ARG if the workspace is too small. */
 int lrstv_zsolve(const float *T, int n1, int n2, int n3, const float w[3], float mu, float *Z,
                  void *workspace, size_t workspace_bytes, void *stream);
 /* t-SVT of a real cube (eq. E_solution with Theorem 4.2's t-SVD): DFT along

@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
   // two shared-memory stages, so that a chunk is staged while the previous
   // chunk's MMAs run, and two TMEM tiles (one per stage)
   constexpr uint32_t kCols = 256;
+  constexpr bool kTwo = KIND == 1 && PREC != 2;  // x - ycoef y; the operators' DFTs take one cube
   constexpr uint32_t kStageBytes = stage_bytes(KIND), kLoB = blocks_b(KIND) * kBlockB;
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tslot;
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
     gK = KIND == 1 ? f.n3 : f.h;
     if (KIND == 1) {
       xb = f.x + (size_t)b * f.N;
-      if (f.y) yb = f.y + (size_t)b * f.N;
+      if (kTwo && f.y) yb = f.y + (size_t)b * f.N;
     } else {
       specb = f.spec + (size_t)b * f.h * f.P;
     }
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
     const int m = am < gM ? am : 0;
     if (KIND == 1) {
       xp = xb + m + as * ak;
-      if (yb) yp = yb + m + as * ak;
+      if (kTwo && yb) yp = yb + m + as * ak;
     } else {
       ap = specb + wpos(m) + as * ak;
     }
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
   float2 ra[kRun], rb[KIND == 0 ? kHalf : 1];
   // KIND 1 with a second cube: its raw values, combined (x - ycoef y) only when
   // the chunk is stored, so that the loads stay in flight meanwhile
-  float2 ry[KIND == 1 ? kRun : 1];
+  float2 ry[kTwo ? kRun : 1];
   auto load_chunk = [&](int k0) {
     if constexpr (KIND == 1) {
       auto pair = [&](const float *q, int i) -> float2 {
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
 #pragma unroll
       for (int i = 0; i < kRun; ++i) {
         ra[i] = pair(xp, i);
-        if (yp) ry[KIND == 1 ? i : 0] = pair(yp, i);
+        if (kTwo && yp) ry[kTwo ? i : 0] = pair(yp, i);
       }
     } else {
       const float2 *q = ap + as * k0;
@@ -361,8 +362,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
 #pragma unroll
     for (int i = 0; i < kRun; ++i) {
       float2 v = ra[i];
-      if (KIND == 1 && yp) {
-        const float2 w = ry[KIND == 1 ? i : 0];
+      if (kTwo && yp) {
+        const float2 w = ry[kTwo ? i : 0];
         v = make_float2(v.x - f.ycoef * w.x, v.y - f.ycoef * w.y);
       }
       if ((KIND == 2 && f.trans) || (KIND == 0 && OPB == 2)) v.y = -v.y;
@@ -546,6 +547,89 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
     if (ok) wait_mmas(last);
     ok = __syncthreads_and(ok) != 0;
     if (ok) drain(last);
+  }
+  if constexpr (PREC == 2) {
+    // Below about 2^-102 the low halves leave FP32's normal range and a value's
+    // digits are lost (2.6e-6 of a cube at 1e-34).  The single operators take any
+    // magnitude: a warp whose part of the tile lies all below what K such terms can
+    // sum to forms it again with FP32 FMAs, eight terms at a time, unless an operand
+    // is zero.  One accumulator decides for most warps: a Z-solve of 145 x 145 x 220
+    // takes 261 us without it and 262 with it (cubes below 1e-30: 2.7 ms, of zeros 390
+    // us); collecting the operands' magnitudes where they are split took 312.
+    constexpr float limit = KIND == 0 ? 0x1p-93f : 0x1p-90f;  // K up to 512, 4096
+    float most = fabsf(accRe[0]);
+    bool low = ok && m0 + row - lane < gM && n0 + colh < gN &&
+               !__any_sync(0xffffffffu, !(most < limit));
+    if (low) {
+#pragma unroll
+      for (int c = 0; c < TN / 2; ++c)
+        most = fmaxf(most, fmaxf(fabsf(accRe[c]), fabsf(accIm[c])));
+      low = !__any_sync(0xffffffffu, !(most < limit));
+    }
+    if (low) {
+      const int gm = m0 + row < gM ? m0 + row : 0, sl = KIND == 0 ? slice_of(gm) : 0;
+      auto at = [&](int k) -> float2 {  // A(gm, k)
+        if constexpr (KIND == 0) {
+          static_assert(OPB != 2, "the operators form no Gram products");
+          return g.A[(size_t)sl * g.sA + row_of(gm) + (size_t)g.lda * k];
+        } else if constexpr (KIND == 1) {
+          return make_float2(f.x[(size_t)blockIdx.z * f.N + gm + f.P * k], 0.f);
+        } else {
+          const float2 v = f.spec[((size_t)blockIdx.z * f.h + k) * f.P + wpos(gm)];
+          return make_float2(v.x, f.trans ? -v.y : v.y);
+        }
+      };
+      auto with = [&](int k, int n) -> float2 {  // op(B)(k, n)
+        if constexpr (KIND == 0) {
+          const float2 v = g.B[(size_t)b * g.sB + (OPB == 1 ? n + (size_t)g.ldb * k
+                                                            : (size_t)g.ldb * n + k)];
+          return make_float2(v.x, OPB == 1 ? -v.y : v.y);
+        } else {
+          const float2 v = f.tw3[(unsigned)n * (unsigned)k % (unsigned)f.n3];
+          if (KIND == 1) return v;
+          const float w = (k == 0 || 2 * k == f.n3) ? 1.0f : 2.0f;
+          return make_float2(w * v.x, -w * v.y);
+        }
+      };
+      bool a_any = false, b_any = KIND != 0;
+      for (int k = 0; k < gK; ++k) {
+        const float2 v = at(k);
+        a_any |= v.x != 0.f || v.y != 0.f;
+        if (KIND == 0 && n0 + colh + lane < gN) {
+          const float2 w = with(k, n0 + colh + lane);
+          b_any |= w.x != 0.f || w.y != 0.f;
+        }
+      }
+      if (__any_sync(0xffffffffu, a_any) && __any_sync(0xffffffffu, b_any)) {
+#pragma unroll
+        for (int c0 = 0; c0 < TN / 2; c0 += 4) {
+          float re[4] = {}, im[4] = {};
+          for (int k0 = 0; k0 < gK; k0 += 8) {
+            float pr[4] = {}, pi[4] = {};
+            for (int k = k0; k < k0 + 8 && k < gK; ++k) {
+              const float2 a = at(k);
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const int n = n0 + colh + c0 + c;
+                const float2 v = with(k, n < gN ? n : 0);
+                pr[c] = fmaf(a.x, v.x, fmaf(-a.y, v.y, pr[c]));
+                pi[c] = fmaf(a.x, v.y, fmaf(a.y, v.x, pi[c]));
+              }
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              re[c] += pr[c];
+              im[c] += pi[c];
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            accRe[c0 + c] = re[c];
+            accIm[c0 + c] = im[c];
+          }
+        }
+      }
+    }
   }
   // give MMAs still in flight a last bounded chance to land before the free
   auto last_wait = [&]() {
@@ -802,6 +886,7 @@ cudaError_t launch_mma_peak(int prec, int nsm, long long n_mma, int *err, cudaSt
 cudaError_t launch_dft3_tc(int kind, const Dft3 &f, int nb, int *err, cudaStream_t st, int prec) {
   if (f.P == 0 || nb <= 0) return cudaSuccess;
   if (f.P > (size_t)TM * 0x7fffffff / 4) return cudaErrorInvalidValue;
+  if (prec == 2 && f.y) return cudaErrorInvalidValue;
   if (kind == 1)
     return prec == 1   ? launch_dft<1, 1>(f, nb, err, st)
            : prec == 2 ? launch_dft<1, 2>(f, nb, err, st)
