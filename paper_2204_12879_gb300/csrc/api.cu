@@ -1181,7 +1181,7 @@ struct BatchGroup {
   int m;              // cubes
   lrstv_plan **pls;   // their plans, in batch order; pls[0] holds the group's block bases
   void *arena;
-  int big;            // slices taller than the common launch takes: one launch
+  int big;            // slices taller than the common launch takes: one launch a cube
 };
 
 struct lrstv_batch {
@@ -1286,7 +1286,7 @@ int group_fs_dual(const BatchGroup &g, cudaStream_t st) {
 
 // Step 4 (E) of every cube: per group the mode-3 DFT, the warm start's
 // products and the RMS norms; one Jacobi launch over the slices of
-// all groups (taller slices: one launch per group); per group sigma and
+// all groups (taller slices: one launch per cube); per group sigma and
 // V diag g, the reconstruction and the inverse DFT with Gamma4.
 int batch_e_step(lrstv_batch *b, cudaStream_t st) {
   const double mu = b->plans[0]->mu;

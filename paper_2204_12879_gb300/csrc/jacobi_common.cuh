@@ -37,21 +37,20 @@ __device__ __forceinline__ float2 ldw(const float2 *p) {
 
 // This thread's share of sum |x_e|^2 over n complex values (e = thread,
 // thread + blockDim.x, ...), in four chains so that four loads are in flight.
-template <bool CG>
 __device__ __forceinline__ float sumsq4(const float2 *x, size_t n) {
   const size_t T = blockDim.x;
   float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;
   size_t e = threadIdx.x;
   for (; e + 3 * T < n; e += 4 * T) {
-    const float2 a = ldw<CG>(x + e), b = ldw<CG>(x + e + T), c = ldw<CG>(x + e + 2 * T),
-                 d = ldw<CG>(x + e + 3 * T);
+    const float2 a = x[e], b = x[e + T], c = x[e + 2 * T],
+                 d = x[e + 3 * T];
     p0 = fmaf(a.x, a.x, fmaf(a.y, a.y, p0));
     p1 = fmaf(b.x, b.x, fmaf(b.y, b.y, p1));
     p2 = fmaf(c.x, c.x, fmaf(c.y, c.y, p2));
     p3 = fmaf(d.x, d.x, fmaf(d.y, d.y, p3));
   }
   for (; e < n; e += T) {
-    const float2 a = ldw<CG>(x + e);
+    const float2 a = x[e];
     p0 = fmaf(a.x, a.x, fmaf(a.y, a.y, p0));
   }
   return (p0 + p1) + (p2 + p3);
@@ -60,14 +59,13 @@ __device__ __forceinline__ float sumsq4(const float2 *x, size_t n) {
 // Per-slice set-up of a packed Jacobi run by the whole CTA: V := I unless warm
 // (warm: V holds the basis W was multiplied by), then ||W||_F^2, returned to
 // every thread (s_red: 32 floats of shared memory).
-template <bool CG>
 __device__ __forceinline__ float pk_setup(int nr, int nc, const float2 *W, float2 *V, int warm,
                                           float *s_red) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (!warm)
     for (int e = tid; e < nc * nc; e += blockDim.x)
       V[e] = make_float2((e % nc) == (e / nc) ? 1.0f : 0.0f, 0.0f);
-  float part = sumsq4<CG>(W, (size_t)nr * nc);
+  float part = sumsq4(W, (size_t)nr * nc);
   part = warp_sum(part);
   if (lane == 0) s_red[warp] = part;
   __syncthreads();

@@ -14,8 +14,8 @@
 //    shared memory, a panel's W and V columns held in registers while later
 //    panels stream past, one column pair per half-warp, paired FP32
 //    instructions (__ffma2_rn) on a split row-pair layout;
-//  - k_jacobi (any nr up to 512): round-robin over all columns in global
-//    memory (L2-resident), one pair per warp.
+//  - k_jacobi (eigen-solves of 257 to 512 rows): round-robin over all columns in
+//    global memory (L2-resident), one pair per warp.
 // The other Fourier slices' SVDs are jacobi_blk.cu's.
 #include <float.h>
 
@@ -25,11 +25,11 @@ namespace lrstv {
 
 namespace {
 
-template <int R>
-__global__ void __launch_bounds__(R <= 8 ? 1024 : 512)
+__global__ void __launch_bounds__(512)
     k_jacobi(int nr, int nc, size_t wstride, size_t vstride, float2 *W_all, float2 *V_all,
              float t, int max_sweeps, float tol, float negl_rel, int *__restrict__ sweeps_out,
              unsigned long long *__restrict__ work, JacOpt o) {
+  constexpr int R = 16;  // rows a lane
   const int warm = o.warm;
   float2 *W = W_all + (size_t)blockIdx.x * wstride;
   float2 *V = V_all + (size_t)blockIdx.x * vstride;
@@ -138,17 +138,7 @@ __global__ void __launch_bounds__(R <= 8 ? 1024 : 512)
     __syncthreads();
   }
 
-  // g_i = max(1 - t / sigma_i, 0); the sigma-vs-t decision is taken in FP64.
-  for (int i = warp; i < nc; i += nwarps) {
-    const float2 *wi = W + (size_t)nr * i;
-    float n2 = 0.f;
-    for (int row = lane; row < nr; row += 32) n2 = fmaf(wi[row].x, wi[row].x, fmaf(wi[row].y, wi[row].y, n2));
-    n2 = warp_sum(n2);
-    const double sigma = sqrt((double)n2);
-    const float g = t < 0.0f ? 1.0f : (sigma > (double)t ? (float)(1.0 - (double)t / sigma) : 0.0f);
-    float2 *vi = V + (size_t)nc * i;
-    for (int row = lane; row < nc; row += 32) vi[row] = make_float2(vi[row].x * g, vi[row].y * g);
-  }
+  pk_epilogue<false>(nr, nc, W, V, t);
   if (tid == 0) sweeps_out[blockIdx.x] = converged ? sweeps : -max_sweeps;
   if (work && lane == 0) {
     atomicAdd(work + 0, n_pairs);
@@ -157,10 +147,8 @@ __global__ void __launch_bounds__(R <= 8 ? 1024 : 512)
 }
 
 // ---------------------------------------------------------------------------
-// Shared pieces of the packed kernel: panel width, rotation formula.
-// Panel width (columns) of the packed kernels: 32 with 16-warp CTAs, or 16
-// with 8-warp CTAs, two of which share an SM (a warp per pair of columns of
-// a panel: PW / 2 warps, PW half-warps).
+// Shared pieces of the packed kernel: panel width (columns; a warp per pair of
+// them), rotation formula.
 constexpr int kPW = 32;
 
 struct Rot {
@@ -168,8 +156,6 @@ struct Rot {
   float d;  // |a'|^2 = |a|^2 - d and |b'|^2 = |b|^2 + d (d = t |g|, the 2x2 Schur rotation's shift)
 };
 
-// Rotation of the 2x2 Hermitian [[al, g], [conj g, be]], or false when the
-// pair is orthogonal to tolerance or a column is negligible.
 // Rotation of the 2x2 Hermitian [[al, g], [conj g, be]], or false when the
 // pair is orthogonal to tolerance (|g|^2 <= tol^2 al be) or a column is
 // negligible.  Unitarity rests on c = 1/sqrt(1 + t^2), s = c t and |e| = 1,
@@ -194,8 +180,7 @@ __device__ __forceinline__ bool make_rot(float al, float be, float gr, float gi,
   return true;
 }
 
-
-constexpr int kHW = kPW / 2;  // warps per CTA of the 32-column packed kernel
+constexpr int kHW = kPW / 2;  // warps per CTA
 
 __device__ __forceinline__ float half_sum(float v) {
 #pragma unroll
@@ -204,7 +189,7 @@ __device__ __forceinline__ float half_sum(float v) {
 }
 
 // ---------------------------------------------------------------------------
-// Packed kernel (nr <= 224): the half-warp panel scheme with Blackwell's
+// Packed kernel (nr <= 256): the half-warp panel scheme with Blackwell's
 // paired FP32 instructions (__ffma2_rn / __fmul2_rn: two FP32 FMAs per lane
 // per instruction).  Staged columns use a split row-pair layout: row pair m is
 // one float4 (re_2m, re_2m+1, im_2m, im_2m+1), so a 128-bit load gives the two
@@ -350,7 +335,7 @@ __device__ __forceinline__ void pk_rot_stream(float4 (&a)[K], float4 *col, const
 
 // Staging of panels into shared memory: a shared panel holds ld2 row pairs
 // per column in the split layout, zero padded, of wcols columns of n rows;
-// warp w copies columns w, w + PW / 2.  A lane's row pairs of one column:
+// warp w copies columns w, w + kHW.  A lane's row pairs of one column:
 // ld2 <= kStageIt * 32 for every packed shape (PkShape: at most 128).
 constexpr int kStageIt = 4;
 
@@ -390,29 +375,27 @@ __device__ __forceinline__ float col_store(float4 *d, const float2 (&x0)[kStageI
 // each) before its first shared store, so that 16 NCOL loads a lane are in
 // flight.  NCOL = 2 holds 32 float2 a lane, for stagings with no register
 // panel live.
-// With a column map (cols, shared memory: the panel's wcols column indices),
-// sW and sV are the slice's first columns and panel column c is column
-// cols[c]; without one the panel's columns are contiguous from sW and sV.
-template <int PW, int NCOL>
+// sW and sV are the slice's first columns; panel column c is column cols[c]
+// (shared memory: the panel's wcols column indices).
+template <int NCOL>
 __device__ __forceinline__ void pk_stage_wv(float4 *dW, const float2 *sW, int nr, float *nrm,
                                             float4 *dV, const float2 *sV, int nc, int ld2,
-                                            int wcols, const int *cols = nullptr) {
-  constexpr int HW = PW / 2;
+                                            int wcols, const int *cols) {
   const int lane = threadIdx.x & 31;
-  for (int c0 = threadIdx.x >> 5; c0 < PW; c0 += NCOL * HW) {
+  for (int c0 = threadIdx.x >> 5; c0 < kPW; c0 += NCOL * kHW) {
     float2 w0[NCOL][kStageIt], w1[NCOL][kStageIt], v0[NCOL][kStageIt], v1[NCOL][kStageIt];
 #pragma unroll
     for (int k = 0; k < NCOL; ++k) {
-      const int c = c0 + k * HW;
-      const bool real = c < PW && c < wcols;
-      const int g = cols ? (real ? cols[c] : 0) : c;
+      const int c = c0 + k * kHW;
+      const bool real = c < kPW && c < wcols;
+      const int g = real ? cols[c] : 0;
       col_load(w0[k], w1[k], sW + (size_t)nr * g, nr, ld2, real);
       col_load(v0[k], v1[k], sV + (size_t)nc * g, nc, ld2, real);
     }
 #pragma unroll
     for (int k = 0; k < NCOL; ++k) {
-      const int c = c0 + k * HW;
-      if (c >= PW) break;
+      const int c = c0 + k * kHW;
+      if (c >= kPW) break;
       const float part = warp_sum(col_store(dW + ld2 * c, w0[k], w1[k], ld2));
       if (lane == 0) nrm[c] = part;
       col_store(dV + ld2 * c, v0[k], v1[k], ld2);
@@ -420,12 +403,11 @@ __device__ __forceinline__ void pk_stage_wv(float4 *dW, const float2 *sW, int nr
   }
 }
 
-template <int PW>
 __device__ __forceinline__ void pk_stage_out(float2 *dst, const float4 *src, int ld2, int n,
-                                             int wcols, const int *cols = nullptr) {
+                                             int wcols, const int *cols) {
   const int lane = threadIdx.x & 31;
-  for (int c = threadIdx.x >> 5; c < wcols; c += PW / 2) {
-    float2 *d = dst + (size_t)n * (cols ? cols[c] : c);
+  for (int c = threadIdx.x >> 5; c < wcols; c += kHW) {
+    float2 *d = dst + (size_t)n * cols[c];
     const float4 *s = src + ld2 * c;
     for (int m = lane; 2 * m < n; m += 32) {
       const float4 v = s[m];
@@ -444,16 +426,16 @@ struct PkShape {
 
 // The pairs inside one staged panel (W in sW with squared norms s_na, V in
 // sVa; wa real columns): 31 rounds of 16 disjoint pairs, one per warp.
-template <int KP, int PW>
+template <int KP>
 __device__ __forceinline__ void pk_intra(float4 *sW, float4 *sVa, float *s_na, int wa, float tol,
                                          float negl, unsigned &n_pairs, unsigned &n_rot,
                                          int &rotated) {
   constexpr int KPF = PkShape<KP>::KPF;
   constexpr int LD2 = PkShape<KP>::LD2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r = 0; r < PW - 1; ++r) {
+  for (int r = 0; r < kPW - 1; ++r) {
     int p, q;
-    pair_of(r, warp, PW, p, q);
+    pair_of(r, warp, kPW, p, q);
     if (p < wa && q < wa) {
       float4 xa[KPF], xb[KPF];
 #pragma unroll
@@ -500,7 +482,7 @@ __device__ __forceinline__ void pk_intra(float4 *sW, float4 *sVa, float *s_na, i
 // which warp w owns streamed columns 2c, 2c+1 (c = (w + R) mod 16) and its
 // half-warps rotate them in swapped order, so only the warp synchronises
 // between the two sub-steps and the block once per double round.
-template <int KP, int PW>
+template <int KP>
 __device__ __forceinline__ void pk_cross_pass(float4 (&aW)[KP], float4 (&aV)[KP], bool mine,
                                               float4 *sW, float4 *sVb, float *s_nb, int wb,
                                               float tol, float negl, unsigned &n_pairs,
@@ -514,9 +496,9 @@ __device__ __forceinline__ void pk_cross_pass(float4 (&aW)[KP], float4 (&aV)[KP]
   // panel (the whole warp shuffles: both halves compute theirs)
   float al_reg = half_sum(pk_norm<KP>(aW));
   __syncthreads();
-  for (int r = 0; r < PW; ++r) {
+  for (int r = 0; r < kPW; ++r) {
     const int sub = r & 1;
-    const int cpi = (warp + (r >> 1)) & (PW / 2 - 1);
+    const int cpi = (warp + (r >> 1)) & (kHW - 1);
     const int j = 2 * cpi + ((unit & 1) ^ sub);
     const bool real = mine && j < wb;
 #pragma unroll
@@ -587,18 +569,18 @@ __device__ __forceinline__ void pk_to_registers(const float4 *sW, const float4 *
 }
 
 // Panel a back to global memory from the registers (W) and, through sVa, V.
-template <int KP, int PW>
+template <int KP>
 __device__ __forceinline__ void pk_from_registers(const float4 (&aW)[KP], const float4 (&aV)[KP],
                                                   bool mine, float4 *sVa, float2 *Wa,
                                                   float2 *Va, int nr, int nc, int wa,
-                                                  const int *cols = nullptr) {
+                                                  const int *cols) {
   constexpr int LD2 = PkShape<KP>::LD2;
   const int unit = threadIdx.x >> 4, ul = threadIdx.x & 15;
 #pragma unroll
   for (int k = 0; k < KP; ++k) sVa[LD2 * unit + ul + 16 * k] = aV[k];
   __syncthreads();
   if (mine) {
-    float2 *wcol = Wa + (size_t)nr * (cols ? cols[unit] : unit);
+    float2 *wcol = Wa + (size_t)nr * cols[unit];
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
       const int m = ul + 16 * k;
@@ -606,7 +588,7 @@ __device__ __forceinline__ void pk_from_registers(const float4 (&aW)[KP], const 
       if (2 * m + 1 < nr) wcol[2 * m + 1] = make_float2(aW[k].y, aW[k].w);
     }
   }
-  pk_stage_out<PW>(Va, sVa, LD2, nc, wa, cols);
+  pk_stage_out(Va, sVa, LD2, nc, wa, cols);
 }
 
 // Columns of a slice of the packed kernels at most (nc <= nr <= 256).
@@ -642,35 +624,35 @@ __device__ void col_norms(int nr, int nc, const float2 *W, float *key) {
   }
 }
 
-// The packed Jacobi SVT of one matrix by the whole CTA (PW / 2 warps): W (nr x
+// The packed Jacobi SVT of one matrix by the whole CTA (kHW warps): W (nr x
 // nc) and V (nc x nc) in global memory, `smem` the CTA's dynamic shared memory
-// (3 PW LD2 float4).  Panel by panel: panel a's own pairs, then panel a (in
+// (3 kPW LD2 float4).  Panel by panel: panel a's own pairs, then panel a (in
 // registers) against every later panel b streamed through shared memory.
 // Writes the sweep count (negative at the cap) to *sweeps_slot.
-template <int KP, int PW>
+template <int KP>
 __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float2 *V, float t,
                                                 int max_sweeps, float tol, float negl_rel,
                                                 int *sweeps_slot, unsigned long long *work,
                                                 float4 *smem, const JacOpt &o, int slice) {
   constexpr int LD2 = PkShape<KP>::LD2;
   float4 *sW = smem;              // panel a (own pairs), then panel b: W
-  float4 *sVa = sW + PW * LD2;    // panel a: V
-  float4 *sVb = sVa + PW * LD2;   // panel b: V
+  float4 *sVa = sW + kPW * LD2;    // panel a: V
+  float4 *sVb = sVa + kPW * LD2;   // panel b: V
   const int tid = threadIdx.x, ul = tid & 15, unit = tid >> 4;
   __shared__ float s_red[32];
   __shared__ int s_rot;
   // squared column norms of panel a and of the streamed panel b: exact when
   // a panel is staged, then carried through each rotation by the 2x2 update
   // (|a|^2 - d, |b|^2 + d), so that a pair's test needs only its inner product
-  __shared__ float s_na[PW], s_nb[PW];
+  __shared__ float s_na[kPW], s_nb[kPW];
   // the sweep's column order (position -> column; panel a holds positions
-  // a PW ...) and each column's squared norm as the sweep left it
+  // a kPW ...) and each column's squared norm as the sweep left it
   __shared__ int s_perm[kSortCols];
   __shared__ float s_key[kSortCols];
 
-  const float fro2 = pk_setup<false>(nr, nc, W, V, o.warm, s_red);
+  const float fro2 = pk_setup(nr, nc, W, V, o.warm, s_red);
   const float negl = negl_rel * fro2;
-  const int npan = (nc + PW - 1) / PW;
+  const int npan = (nc + kPW - 1) / kPW;
   unsigned n_pairs = 0, n_rot = 0;  // lane 0 (own pairs) and ul 0 (cross pairs) count
   int sweeps = (nc < 2) ? 1 : 0;
   bool converged = (nc < 2);
@@ -700,29 +682,29 @@ __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float
     if (tid == 0) s_rot = 0;
     int rotated = 0;
     for (int a = 0; a < npan; ++a) {
-      const int ca = a * PW, wa = min(PW, nc - ca);
+      const int ca = a * kPW, wa = min(kPW, nc - ca);
       const int *cola = s_perm + ca;  // panel a: positions ca ... of the sweep's order
       __syncthreads();
-      pk_stage_wv<PW, 2>(sW, W, nr, s_na, sVa, V, nc, LD2, wa, cola);
+      pk_stage_wv<2>(sW, W, nr, s_na, sVa, V, nc, LD2, wa, cola);
       __syncthreads();
-      pk_intra<KP, PW>(sW, sVa, s_na, wa, tol, negl, n_pairs, n_rot, rotated);
+      pk_intra<KP>(sW, sVa, s_na, wa, tol, negl, n_pairs, n_rot, rotated);
       if (tid < wa) s_key[cola[tid]] = s_na[tid];
       const bool mine = unit < wa;
       pk_to_registers<KP>(sW, sVa, aW, aV);
       for (int b = a + 1; b < npan; ++b) {
-        const int cb = b * PW, wb = min(PW, nc - cb);
+        const int cb = b * kPW, wb = min(kPW, nc - cb);
         const int *colb = s_perm + cb;
         __syncthreads();
-        pk_stage_wv<PW, 1>(sW, W, nr, s_nb, sVb, V, nc, LD2, wb, colb);
+        pk_stage_wv<1>(sW, W, nr, s_nb, sVb, V, nc, LD2, wb, colb);
         float al = 0.0f;
-        pk_cross_pass<KP, PW>(aW, aV, mine, sW, sVb, s_nb, wb, tol, negl, n_pairs, n_rot, rotated,
+        pk_cross_pass<KP>(aW, aV, mine, sW, sVb, s_nb, wb, tol, negl, n_pairs, n_rot, rotated,
                               &al);
         if (mine && ul == 0) s_key[cola[unit]] = al;
         if (tid < wb) s_key[colb[tid]] = s_nb[tid];
-        pk_stage_out<PW>(W, sW, LD2, nr, wb, colb);
-        pk_stage_out<PW>(V, sVb, LD2, nc, wb, colb);
+        pk_stage_out(W, sW, LD2, nr, wb, colb);
+        pk_stage_out(V, sVb, LD2, nc, wb, colb);
       }
-      pk_from_registers<KP, PW>(aW, aV, mine, sVa, W, V, nr, nc, wa, cola);
+      pk_from_registers<KP>(aW, aV, mine, sVa, W, V, nr, nc, wa, cola);
     }
     if (rotated) s_rot = 1;
     __syncthreads();
@@ -740,16 +722,15 @@ __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float
   }
 }
 
-// Slices of up to 64 rows fit in 64 registers a thread, and 16-column panels
-// take 8-warp CTAs: two CTAs share an SM.
-template <int KP, int PW>
-__global__ void __launch_bounds__(PW * 16, (KP <= 2 || PW == 16) ? 2 : 1)
+// Slices of up to 64 rows fit in 64 registers a thread: two CTAs share an SM.
+template <int KP>
+__global__ void __launch_bounds__(kPW * 16, KP <= 2 ? 2 : 1)
     k_jacobi_pk(int nr, int nc, size_t wstride, size_t vstride, float2 *W_all, float2 *V_all,
                 float t, int max_sweeps, float tol, float negl_rel, int *__restrict__ sweeps_out,
                 unsigned long long *__restrict__ work, JacOpt o) {
   extern __shared__ float4 smem_f4[];
   const int s = blockIdx.x;
-  jacobi_pk_slice<KP, PW>(nr, nc, W_all + (size_t)s * wstride, V_all + (size_t)s * vstride, t,
+  jacobi_pk_slice<KP>(nr, nc, W_all + (size_t)s * wstride, V_all + (size_t)s * vstride, t,
                           max_sweeps, tol, negl_rel, sweeps_out + s, work, smem_f4, o, s);
 }
 
@@ -758,10 +739,10 @@ cudaError_t launch_pk(int nslices, int nr, int nc, size_t ws, size_t vs, float2 
                       float t, int max_sweeps, float tol, float negl, int *sweeps,
                       unsigned long long *work, const JacOpt &o, cudaStream_t st) {
   const size_t smem = sizeof(float4) * 3 * (size_t)kPW * PkShape<KP>::LD2;
-  cudaError_t e = cudaFuncSetAttribute(k_jacobi_pk<KP, kPW>,
+  cudaError_t e = cudaFuncSetAttribute(k_jacobi_pk<KP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_jacobi_pk<KP, kPW><<<nslices, kPW * 16, smem, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol,
+  k_jacobi_pk<KP><<<nslices, kPW * 16, smem, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol,
                                                         negl, sweeps, work, o);
   return cudaGetLastError();
 }
@@ -805,7 +786,7 @@ __global__ void __launch_bounds__(1024)
                 unsigned *__restrict__ gmax) {
   __shared__ float s_red[32];
   const float2 *Ws = W + (size_t)blockIdx.x * wstride;
-  float part = sumsq4<false>(Ws, (size_t)nr * nc);
+  float part = sumsq4(Ws, (size_t)nr * nc);
   part = warp_sum(part);
   if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = part;
   __syncthreads();
@@ -952,16 +933,12 @@ cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, floa
   const bool eig = o.negl_rel >= 0.0f;
   if (!eig && (o.sched || nr > 256))
     return launch_jacobi_blk(d, nslices, W, V, t, max_sweeps, sweeps, work, st, o);
-  const int np = nc + (nc & 1);
-  const int R = (nr + 31) / 32;
-  int pairs = np / 2 < 1 ? 1 : np / 2;
-  const int maxw = R <= 8 ? 32 : 16;
-  const int nw = pairs < maxw ? pairs : maxw;
+  const int pairs = (nc + 1) / 2, nw = pairs < 16 ? pairs : 16;  // k_jacobi's warps
   const float eps = FLT_EPSILON * 0.5f;
   const float tol = jacobi_tol0(nr), negl = eig ? o.negl_rel : ((float)nr * eps) * ((float)nr * eps);
   const size_t ws = d.P, vs = (size_t)nc * nc;
   if (nr <= 256) {
-    const int KP = R;
+    const int KP = (nr + 31) / 32;
 #define LRSTV_PK(K) \
   return launch_pk<K>(nslices, nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o, st)
     if (KP <= 1) LRSTV_PK(1);
@@ -972,13 +949,8 @@ cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, floa
     LRSTV_PK(8);
 #undef LRSTV_PK
   }
-  dim3 grid(nslices), block(32 * nw);
-  if (R <= 1) k_jacobi<1><<<grid, block, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
-  else if (R <= 2) k_jacobi<2><<<grid, block, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
-  else if (R <= 4) k_jacobi<4><<<grid, block, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
-  else if (R <= 8) k_jacobi<8><<<grid, block, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
-  else if (R <= 16) k_jacobi<16><<<grid, block, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
-  else return cudaErrorInvalidValue;
+  if (nr > 512) return cudaErrorInvalidValue;
+  k_jacobi<<<nslices, 32 * nw, 0, st>>>(nr, nc, ws, vs, W, V, t, max_sweeps, tol, negl, sweeps, work, o);
   return cudaGetLastError();
 }
 

@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
       const int gm = m0 + row < gM ? m0 + row : 0, sl = KIND == 0 ? slice_of(gm) : 0;
       auto at = [&](int k) -> float2 {  // A(gm, k)
         if constexpr (KIND == 0) {
-          static_assert(OPB != 2, "the operators form no Gram products");
+          static_assert(OPB == 0, "of the operators' products");
           return g.A[(size_t)sl * g.sA + row_of(gm) + (size_t)g.lda * k];
         } else if constexpr (KIND == 1) {
           return make_float2(f.x[(size_t)blockIdx.z * f.N + gm + f.P * k], 0.f);
@@ -581,9 +581,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
       };
       auto with = [&](int k, int n) -> float2 {  // op(B)(k, n)
         if constexpr (KIND == 0) {
-          const float2 v = g.B[(size_t)b * g.sB + (OPB == 1 ? n + (size_t)g.ldb * k
-                                                            : (size_t)g.ldb * n + k)];
-          return make_float2(v.x, OPB == 1 ? -v.y : v.y);
+          return g.B[(size_t)b * g.sB + (size_t)g.ldb * n + k];
         } else {
           const float2 v = f.tw3[(unsigned)n * (unsigned)k % (unsigned)f.n3];
           if (KIND == 1) return v;
@@ -852,7 +850,8 @@ cudaError_t launch_prec(const CGemm &g, int *err, cudaStream_t st) {
   }
   if (g.opB == 0 && g.epi == 0) return launch_one<0, 0, PREC>(g, err, st);
   if (g.opB == 0 && g.epi == 1) return launch_one<0, 1, PREC>(g, err, st);
-  if (g.opB == 1 && g.epi == 0) return launch_one<1, 0, PREC>(g, err, st);
+  if constexpr (PREC != 2)  // the operators' reconstruction is in FP32
+    if (g.opB == 1 && g.epi == 0) return launch_one<1, 0, PREC>(g, err, st);
   return cudaErrorInvalidValue;
 }
 
