@@ -236,17 +236,6 @@ def jacobi_flops(prof, shape):
     return 8.0 * nr * prof.jacobi_pairs + 18.0 * (nr + nc) * prof.jacobi_rotations
 
 
-def jacobi_textbook_flops(prof, shape):
-    """The same launches at the usual count of a complex one-sided Jacobi
-    sweep, about 30 n^3 flops a slice (n = nc; pairs, their inner products and
-    rotations of W and V), times the sweep-slices the launches ran (pairs
-    examined / (nc (nc - 1) / 2))."""
-    n1, n2, _ = shape
-    nc = min(n1, n2)
-    sweep_slices = prof.jacobi_pairs / max(nc * (nc - 1) / 2, 1)
-    return 30.0 * nc ** 3 * sweep_slices
-
-
 def derived_peaks(pk, pk_kind, probes, sm_count):
     """The roofs the line's fractions use.  FP32 FMA and TF32 come from this
     run's probes when they ran (the larger of the scalar and paired FMA
@@ -530,14 +519,11 @@ def run_ours(args, wl_name):
     avg_s = kernels[dom]["ms_per_launch"] / 1e3
     if dom == "jacobi":
         flops = jacobi_flops(prof, shape) / prof.launches[6]
-        textbook = jacobi_textbook_flops(prof, shape) / prof.launches[6]
         roof = {"bound": "alu", "achieved": flops / avg_s / 1e12, "peak": peak["fp32"],
                 "unit": "TFLOP/s", "peak_source": peak["fp32_source"],
                 "work": "a column Jacobi's: 8 nr flops per examined column pair, 18 (nr + nc) per "
                         "rotated pair, counted on the device (the kernel forms most of them "
-                        "on the tensor cores)",
-                "achieved_textbook": textbook / avg_s / 1e12,
-                "frac_textbook": textbook / avg_s / 1e12 / peak["fp32"]}
+                        "on the tensor cores: the fraction compares algorithms, not pipes)"}
     else:
         bound, work = kernel_work(dom, shape)
         if bound == "hbm":
@@ -572,6 +558,9 @@ def run_ours(args, wl_name):
                    "mode3_dft": "tensor cores" if args.dft == "tc" else "SIMT direct sums",
                    "jacobi_schedule": "panel-pair tasks of every slice from one queue, on all SMs",
                    "jacobi_panel": 16,
+                   "given_without_effect": [f for f, on in (
+                       ("--jacobi-schedule slice", args.jacobi_schedule == "slice"),
+                       ("--jacobi-panel 16", args.jacobi_panel == 16)) if on],
                    "jacobi_order": ("columns by norm, largest first, from the start"
                                     if args.jacobi_order == "sorted" else "stored order"),
                    "l_update": ("Tucker projection, one HOOI sweep per iteration, ranks %s" % (ranks,)
