@@ -24,7 +24,12 @@
 // and form hi*hi + hi*lo + lo*hi with FP32 accumulation (the Gram adds lo*lo).
 // W is scaled by a power of two that puts ||W||_F into [2^14, 2^15), V by 2^13
 // and Q - I by 2^14, so that no half overflows and the low halves of every
-// column that is not negligible stay above FP16's smallest step.  The tensor
+// column that is not negligible stay above FP16's smallest step.  Between two
+// tasks W and V are held in these halves alone: 22 bits, down to 2^-39 of ||W||_F
+// (2^-38 in V), rounded once for each task that rotates the column, where FP32
+// rotations on the columns round at each of their 16 to 31.  The t-SVT's error
+// against FP64 is 0.60 to 0.90 of what such rotations left (22 cubes of 27 to 91
+// pixels).  A slice that rotates nothing keeps its FP32 values.  The tensor
 // core truncates its sums; the identity is added outside of it, in FP32, so
 // that the truncation is relative to a task's change and does not shorten the
 // columns task after task.  A rotation is applied as a' = a + m a - sigma b,
@@ -192,9 +197,9 @@ __device__ __forceinline__ int pair_index(int np, int r, int p) {
 // both of its panels have had their task of the round before (an arrival
 // each, counted from one sweep to the next: ready on every second one); a sweep's
 // round 0 starts when every task of the sweep before is done.  A task is done
-// for this when W is: V, which nothing but the panels' next V update reads,
-// follows in the order of the panels' tasks (vdone), off the slice's critical
-// path.
+// for this when W is and the panels' V of the tasks before (vdone): V, which
+// nothing but the panels' next V update reads, follows a round behind, and is
+// waited for only when a round's W overtakes the V of the round before.
 struct Sched {
   int *head, *tail, *finished, *err, *npend, *pend_head, *live;
   int *sweep, *left, *pend, *packed;
