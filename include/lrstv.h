@@ -343,8 +343,9 @@ int lrstv_denoise(const float *Y, int n1, int n2, int n3, const lrstv_params *pa
  *          may differ.  Parameters are fixed when the batch is created.
  * The batch owns one plan per cube (lrstv_batch_plan lends it for stats and
  * state export; do not destroy it or change its parameters), one allocation
- * per group and one small allocation for the work list and the task queue.  Slices taller than
- * 256 rows (max(n1, n2)) take a separate Jacobi launch per cube.  The
+ * per group and one small allocation for the work list and the task queue.  Slices
+ * taller than 256 rows (max(n1, n2)) take a separate Jacobi launch per cube, slices
+ * of few columns (min(n1, n2) up to 12, or 16 of up to 48 rows) one per group.  The
  * Jacobi launch is recorded in cube 0's profile (lrstv_profile_*), a
  * group's other launches in the profile of its first cube.  A cube whose plan
  * has the Tucker L-update (lrstv_plan_set_tucker) takes its own launches for
@@ -402,7 +403,8 @@ int lrstv_zsolve(const float *T, int n1, int n2, int n3, const float w[3], float
  * down to 2^-39 of a slice's norm) and holds a slice's factors in them between
  * rotations; angles and sums are FP32.  The result is 2e-6 to 7e-6 relative off
  * the FP64 one for cubes of 24 to 92 pixels a side, set by the sweeps' stopping
- * tolerance.  With a workspace that holds the spectra, V and the counts alone (as
+ * tolerance.  Slices of few columns (see lrstv_batch) run in FP32, one CTA each.
+ * With a workspace that holds the spectra, V and the counts alone (as
  * lrstv_tsvt_noalloc's scratch does) slices of up to 256 rows run in FP32 instead,
  * one CTA each (75 x 91 x 220: 1.4 ms instead of 0.95; 3e-6 to 9e-6 off). */
 int lrstv_tsvt(const float *A, int n1, int n2, int n3, float t, float *out, void *workspace,

@@ -1181,7 +1181,7 @@ struct BatchGroup {
   int m;              // cubes
   lrstv_plan **pls;   // their plans, in batch order; pls[0] holds the group's block bases
   void *arena;
-  int big;            // slices taller than the common launch takes: one launch a cube
+  int alone;          // not in the common Jacobi launch: taller (a launch a cube) or of few columns (one)
 };
 
 struct lrstv_batch {
@@ -1237,6 +1237,9 @@ int task_cmp(const void *x, const void *y) {
   return a->W < b->W ? -1 : (a->W > b->W ? 1 : 0);  // a fixed order among equals
 }
 
+// whether a cube's slices are in the batch's common Jacobi launch
+bool in_common(const Dims &d) { return d.nr <= kBatchMaxNr && !jacobi_few(d.nr, d.nc); }
+
 bool group_tucker(const BatchGroup &g) {
   for (int i = 0; i < g.m; ++i)
     if (g.pls[i]->tucker) return true;
@@ -1286,7 +1289,7 @@ int group_fs_dual(const BatchGroup &g, cudaStream_t st) {
 
 // Step 4 (E) of every cube: per group the mode-3 DFT, the warm start's
 // products and the RMS norms; one Jacobi launch over the slices of
-// all groups (taller slices: one launch per cube); per group sigma and
+// all groups (taller slices: one launch per cube, few columns: per group); per group sigma and
 // V diag g, the reconstruction and the inverse DFT with Gamma4.
 int batch_e_step(lrstv_batch *b, cudaStream_t st) {
   const double mu = b->plans[0]->mu;
@@ -1307,6 +1310,41 @@ int batch_e_step(lrstv_batch *b, cudaStream_t st) {
                            (float)(p->prm.alpha / mu), p->ms2, d.h, p->gemm_err, st));
     }
   }
+  // a group outside of the common launch; few columns need no queue: its cubes are
+  // one batch of slices
+  auto few = [](const BatchGroup &g) { return jacobi_few(g.pls[0]->d.nr, g.pls[0]->d.nc); };
+  auto alone = [&](const BatchGroup &g, cudaStream_t s) -> int {
+    const int n = few(g) ? g.m : 1;
+    for (int i = 0; i < g.m; i += n) {
+      lrstv_plan *p = g.pls[i];
+      Span sp(&p->prof, LRSTV_K_JACOBI, s);
+      JacOpt o;
+      o.conv = wflag && plan_gemm(p).tc ? p->gconv : nullptr;
+      o.warm = warm;
+      o.t_svt = (float)(p->prm.alpha / mu);
+      o.ms2 = p->ms2;
+      o.group = p->d.h;
+      o.sched = p->jsched;
+      o.sort = plan_sort(p);
+      CK(launch_jacobi(p->d, 3 * p->d.h * n, p->specA, p->V, wflag ? -1.0f : o.t_svt, kMaxSweeps,
+                       p->sweeps, p->prof.on ? p->prof.d_work : nullptr, s, o));
+    }
+    return LRSTV_OK;
+  };
+  int rc;
+  // few columns are a chain of latencies on few SMs: beside the common launch, on the
+  // group's side stream (four cubes of 16 x 16 x 4 with four of 64 x 64 x 31, 12
+  // iterations: 8.4 ms, 9.0 in turn)
+  const bool beside = b->ntasks > 0;
+  for (int k = 0; beside && k < b->ngroups; ++k) {
+    const BatchGroup &g = b->groups[k];
+    if (!g.alone || !few(g)) continue;
+    lrstv_plan *p = g.pls[0];
+    CK(cudaEventRecord(p->ev_fs, st));
+    CK(cudaStreamWaitEvent(p->side, p->ev_fs, 0));
+    if ((rc = alone(g, p->side)) != LRSTV_OK) return rc;
+    CK(cudaEventRecord(p->ev_side, p->side));
+  }
   if (b->ntasks > 0) {
     Prof *prof = &b->plans[0]->prof;
     Span sp(prof, LRSTV_K_JACOBI, st);
@@ -1316,21 +1354,11 @@ int batch_e_step(lrstv_batch *b, cudaStream_t st) {
   }
   for (int k = 0; k < b->ngroups; ++k) {
     const BatchGroup &g = b->groups[k];
-    if (!g.big) continue;
-    for (int i = 0; i < g.m; ++i) {
-      lrstv_plan *p = g.pls[i];
-      Span sp(&p->prof, LRSTV_K_JACOBI, st);
-      JacOpt o;
-      o.conv = wflag && plan_gemm(p).tc ? p->gconv : nullptr;
-      o.warm = warm;
-      o.t_svt = (float)(p->prm.alpha / mu);
-      o.ms2 = p->ms2;
-      o.group = p->d.h;
-      o.sched = p->jsched;
-      o.sort = plan_sort(p);
-      CK(launch_jacobi(p->d, 3 * p->d.h, p->specA, p->V, wflag ? -1.0f : o.t_svt, kMaxSweeps,
-                       p->sweeps, p->prof.on ? p->prof.d_work : nullptr, st, o));
-    }
+    if (!g.alone) continue;
+    if (beside && few(g))
+      CK(cudaStreamWaitEvent(st, g.pls[0]->ev_side, 0));
+    else if ((rc = alone(g, st)) != LRSTV_OK)
+      return rc;
   }
   for (int k = 0; k < b->ngroups; ++k) {
     const BatchGroup &g = b->groups[k];
@@ -1442,7 +1470,7 @@ int batch_groups(lrstv_batch *b, const int *dims, const lrstv_params *params) {
       g.pls[i]->own_arena = 0;
     }
     rc = arena_start(g.pls[0], g.arena, bytes);
-    g.big = g.pls[0]->d.nr > kBatchMaxNr;
+    g.alone = !in_common(g.pls[0]->d);
   }
   delete[] gid;
   delete[] cnt;
@@ -1487,7 +1515,7 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
   int ntasks = 0, maxnr = 1, maxnc = 1;
   for (int i = 0; i < ncubes; ++i) {
     const Dims &d = b->plans[i]->d;
-    if (d.nr <= kBatchMaxNr) {
+    if (in_common(d)) {
       ntasks += 3 * d.h;
       if (d.nr > maxnr) maxnr = d.nr;
       if (d.nc > maxnc) maxnc = d.nc;
@@ -1504,7 +1532,7 @@ int lrstv_batch_create(int ncubes, const int *dims, const lrstv_params *params,
     for (int i = 0; i < ncubes; ++i) {
       lrstv_plan *pl = b->plans[i];
       const Dims &d = pl->d;
-      if (d.nr > kBatchMaxNr) continue;
+      if (!in_common(d)) continue;
       for (int s = 0; s < 3 * d.h; ++s) {
         h[k].W = pl->specA + (size_t)s * d.P;
         h[k].V = pl->V + (size_t)s * d.nc * d.nc;

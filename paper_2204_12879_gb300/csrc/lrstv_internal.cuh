@@ -164,8 +164,9 @@ struct JacOpt {
   int group = 1;
   float negl_rel = -1.0f;
   // scratch of jacobi_task_ints(nslices, nc, nslices jacobi_op_bytes(nr, nc))
-  // ints: with it, every SM takes tasks of any slice from a queue (blocked kernel);
-  // without it, one CTA runs a slice (up to 256 rows on the FP32 kernel)
+  // ints: with it, every SM takes tasks of any slice from a queue (blocked kernel,
+  // but for few columns); without it, one CTA runs a slice (up to 256 rows on the
+  // FP32 kernel)
   int *sched = nullptr;
   // nslices flags of launch_gram_check (may be null): a slice whose flag is
   // set ends after one sweep without running it (that sweep would rotate
@@ -196,8 +197,10 @@ cudaError_t launch_gram_check(const Dims &d, int nslices, const float2 *W, float
 // nc, 0) ints).
 size_t jacobi_op_bytes(int nr, int nc);
 size_t jacobi_task_ints(int nslices, int nc, size_t op_total);
+// Whether slices have so few columns that the FP32 kernels take them.
+bool jacobi_few(int nr, int nc);
 // The blocked kernel (jacobi_blk.cu), or the per-slice FP32 kernels (svt.cu): for
-// slices of up to 256 rows without a queue's scratch, and when negl_rel is given
+// slices of few columns, of up to 256 rows without a queue's scratch, and when negl_rel is given
 // (the Tucker eigen-solves, whose null-space columns the blocked kernel's FP16
 // halves would not resolve).
 cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, float t,
@@ -233,7 +236,7 @@ struct SliceTask {
   char *op;          // the slice's operands (jacobi_op_bytes, 256-byte aligned)
 };
 // Largest slice height of a batch's common launch (taller slices would leave
-// one CTA to an SM for all of them).
+// one CTA to an SM for all of them); slices of few columns are not in it either.
 constexpr int kBatchMaxNr = 256;
 // The blocked Jacobi over a list of slices of any shapes up to max_nr x max_nc.
 // warm: as launch_jacobi; keep: V left unscaled (threshold taken as negative);

@@ -1,8 +1,8 @@
 // svt.cu -- the small kernels around the t-SVT's Jacobi (arXiv 2204.12879, eq.
 // E_solution; the slice-wise form follows Theorem 4.2's t-SVD): the RMS norms,
-// the Gram pre-check, sigma and V diag g; and the FP32 one-sided Jacobi of the
-// calls without a task queue's scratch (slices of up to 256 rows, one CTA each) and
-// of the Tucker L-update's eigen-solves.
+// the Gram pre-check, sigma and V diag g; and the FP32 one-sided Jacobi of slices
+// with few columns, of the calls without a task queue's scratch (slices of up to 256
+// rows) and of the Tucker L-update's eigen-solves, one CTA each.
 //
 // The FP32 Jacobi orthogonalises a working matrix W (nr x nc complex, nr >= nc)
 // by one-sided (Hestenes) rotations of column pairs (p, q) until
@@ -14,8 +14,8 @@
 //    shared memory, a panel's W and V columns held in registers while later
 //    panels stream past, one column pair per half-warp, paired FP32
 //    instructions (__ffma2_rn) on a split row-pair layout;
-//  - k_jacobi (eigen-solves of 257 to 512 rows): round-robin over all columns in
-//    global memory (L2-resident), one pair per warp.
+//  - k_jacobi (257 to 512 rows): round-robin over all columns in global memory
+//    (L2-resident), one pair per warp.
 // The other Fourier slices' SVDs are jacobi_blk.cu's.
 #include <float.h>
 
@@ -24,6 +24,21 @@
 namespace lrstv {
 
 namespace {
+
+// Whether a slice needs no sweep, with the sweeps to report: every singular value
+// is at most ||W||_F, so at or below the threshold the SVT is zero whatever the
+// sweeps would find (0); or the Gram check showed that one would rotate no pair (1).
+__device__ __forceinline__ bool slice_known(float fro2, const JacOpt &o, int slice, int &sweeps) {
+  if (o.t_svt >= 0.0f && fro2 <= o.t_svt * o.t_svt) {
+    sweeps = 0;
+    return true;
+  }
+  if (o.conv && o.conv[slice]) {
+    sweeps = 1;
+    return true;
+  }
+  return false;
+}
 
 __global__ void __launch_bounds__(512)
     k_jacobi(int nr, int nc, size_t wstride, size_t vstride, float2 *W_all, float2 *V_all,
@@ -57,13 +72,14 @@ __global__ void __launch_bounds__(512)
     if (lane == 0) s_red[0] = v;
   }
   __syncthreads();
-  const float negl = negl_rel * s_red[0];
+  const float fro2 = s_red[0], negl = negl_rel * fro2;
 
   const int np = nc + (nc & 1);
   unsigned long long n_pairs = 0, n_rot = 0;  // counted by lane 0 of each warp
   // a slice with fewer than two columns is diagonal already: one empty sweep
   int sweeps = (nc < 2) ? 1 : 0;
-  bool converged = (nc < 2);
+  bool converged = slice_known(fro2, o, blockIdx.x, sweeps) || nc < 2;
+  tol = pk_tolerance(tol, fro2, nc, o.t_svt, o.ms2 ? o.ms2[blockIdx.x / o.group] : -1.0f);
   for (int sweep = 1; sweep <= max_sweeps && !converged; ++sweep) {
     if (tid == 0) s_rot = 0;
     __syncthreads();
@@ -655,18 +671,7 @@ __device__ __forceinline__ void jacobi_pk_slice(int nr, int nc, float2 *W, float
   const int npan = (nc + kPW - 1) / kPW;
   unsigned n_pairs = 0, n_rot = 0;  // lane 0 (own pairs) and ul 0 (cross pairs) count
   int sweeps = (nc < 2) ? 1 : 0;
-  bool converged = (nc < 2);
-  // every singular value is at most ||W||_F: at or below the threshold the SVT
-  // is zero whatever the sweeps would find, so none is run
-  if (o.t_svt >= 0.0f && fro2 <= o.t_svt * o.t_svt) {
-    sweeps = 0;
-    converged = true;
-  }
-  // the Gram check showed that a sweep would rotate no pair
-  if (!converged && o.conv && o.conv[slice]) {
-    sweeps = 1;
-    converged = true;
-  }
+  bool converged = slice_known(fro2, o, slice, sweeps) || nc < 2;
   tol = pk_tolerance(tol, fro2, nc, o.t_svt, o.ms2 ? o.ms2[slice / o.group] : -1.0f);
   float4 aW[KP], aV[KP];
   if (!converged) {  // the first sweep's order: by the columns' norms, or as stored
@@ -888,6 +893,14 @@ cudaError_t launch_group_ms2(const Dims &d, int nslices, const float2 *W, int gr
   return cudaGetLastError();
 }
 
+// A slice of one panel of 16 columns, or little more than half of one, is a chain of
+// single tasks, a set-up and a closing launch that the FP32 kernels do in one.  t-SVT
+// with the blocked / the FP32 kernel, us: 20 x 4 x 4 111 / 62, 64 x 12 x 64 156 / 121,
+// 256 x 8 x 64 170 / 121, 512 x 4 x 4 131 / 53.  The ratio at the line, with 4, 31 and
+// 128 bands: 48 x 16 1.15, 0.99, 1.10; 128 x 14 1.08, 1.20, 1.01; 230 x 12 1.02, 1.05,
+// 0.97; beyond it 128 x 16 0.90, 0.90, 1.01; 230 x 13 0.89, 0.96, 0.99.
+bool jacobi_few(int nr, int nc) { return nr > 256 ? nc <= 12 : 48 * nc <= 816 - nr; }
+
 float jacobi_tol0(int nr) { return 8.0f * sqrtf((float)nr) * (FLT_EPSILON * 0.5f); }
 
 cudaError_t launch_gram_check(const Dims &d, int nslices, const float2 *W, float2 *G,
@@ -925,13 +938,13 @@ cudaError_t launch_jacobi(const Dims &d, int nslices, float2 *W, float2 *V, floa
                           cudaStream_t st, const JacOpt &o) {
   const int nr = d.nr, nc = d.nc;
   if (nslices <= 0) return cudaSuccess;
-  // Without a queue's scratch one CTA runs a slice: up to 256 rows the FP32 kernel,
+  // Few columns, or no queue's scratch: one CTA runs a slice.  Without scratch, up to 256 rows the FP32 kernel,
   // which keeps a panel in registers while the others stream past (200 x 200 x 80:
   // 10.5 ms a t-SVT against 23.3 with the blocked kernel's tasks one after another,
   // 64 x 64 x 31: 0.68 against 0.82, 32 x 32 x 16: 0.23 against 0.21); above, the
   // blocked one (280 x 300 x 31: 53 ms against k_jacobi's 84).
   const bool eig = o.negl_rel >= 0.0f;
-  if (!eig && (o.sched || nr > 256))
+  if (!eig && !jacobi_few(nr, nc) && (o.sched || nr > 256))
     return launch_jacobi_blk(d, nslices, W, V, t, max_sweeps, sweeps, work, st, o);
   const int pairs = (nc + 1) / 2, nw = pairs < 16 ? pairs : 16;  // k_jacobi's warps
   const float eps = FLT_EPSILON * 0.5f;
