@@ -98,7 +98,7 @@ cudaError_t launch_cgemm(const CGemm &g, cudaStream_t st);
 // The same GEMM on the tensor cores (tcgen05): prec 0 splits FP32 operands
 // into two TF32 halves (3xTF32, FP32-accurate), prec 1 into two BF16 halves
 // (3xBF16, about 2^-17 relative error per term, the mixed-precision mode); prec
-// 2 is prec 0 for callers without an error slot.
+// 2 is prec 0 with the small split products summed first (more accurate).
 // *err (may be null) is set to 1 if a CTA's wait for its MMAs runs out; its tile
 // is left as it was, or NaN with prec 2.
 cudaError_t launch_cgemm_tc(const CGemm &g, int *err, cudaStream_t st, int prec = 0);
@@ -284,7 +284,7 @@ struct Prof;  // per-kernel event profiler of a plan; null: not profiled
 // Which GEMM implementation a call uses: the tensor cores (with an error
 // slot for bounded-wait timeouts) or the FP32 SIMT kernel.
 constexpr GemmSel kSimt = {false, nullptr, 0, false};
-// the single operators' (lrstv_zsolve, lrstv_tsvt): tensor cores, no error slot
+// the single operators' (lrstv_zsolve, lrstv_tsvt): tensor cores, small products first
 constexpr GemmSel kOperator = {true, nullptr, 2, true};
 cudaError_t gemm(const CGemm &g, GemmSel gs, cudaStream_t st);
 

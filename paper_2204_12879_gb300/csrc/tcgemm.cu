@@ -15,14 +15,12 @@
 // drain into FP32 register accumulators: accumulation error then grows over
 // 16 terms, not over the whole K.
 //
-// What is left of the truncation is that of the sums that hold a hi*hi product: a
-// chunk's four small products are formed first, so that only the two hi*hi are
-// added to a full-size sum instead of all six.  Every such sum shrinks a little, and
-// the shrinking adds up over a run: X of a denoise of 32 x 32 x 16, 20 iterations,
-// is 1.55e-6 off against FP64, 3.52e-6 with hi*hi first (geometric mean of 24 noise
-// seeds), the unrolled X of 64 x 64 x 31 3.2e-7 against 6.1e-7; the instructions and
-// their time are the same.  A Z-solve of 145 x 145 x 220: 4.4e-7 relative,
-// 8.9e-7 with hi*hi first, 1.12e-6 with FP32 FMAs (857 -> 281 us).
+// The tensor core's truncation is then that of the hi*hi sums at each of the six
+// products.  prec = 2 forms a chunk's four small products first, so that only the
+// two hi*hi are added to a full-size sum: for the single operators, whose error
+// against FP64 this keeps below that of FP32 sums (Z-solve of 145 x 145 x 220:
+// 4.4e-7 relative, 8.9e-7 with prec = 0, 1.12e-6 with FP32 FMAs; 857 -> 281 us).  The iterations keep prec =
+// 0, whose rounding their runs' results have always had.
 //
 // Complex arithmetic as real GEMMs with K doubled: for a K chunk,
 //   Re C += [Re A | Im A] . [Re B | -Im B]^T,   Im C += [Re A | Im A] . [Im B | Re B]^T.
@@ -429,8 +427,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
     // Re C (tile columns 0..63) and Im C (64..127) from one N = 128 MMA over two
     // adjacent blocks, so that A is read once for both; the real part alone (KIND 2)
     // from N = 64.  j: A's real parts (KIND 1: the first bands), then the others.
-    // Three split products each, into a fresh tile per chunk, the small ones first
-    // (3xBF16: what it drops hides the difference).
+    // Three split products each, into a fresh tile per chunk.
     const uint32_t id = KIND == 2 ? idesc : idesc2;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -438,11 +435,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_cgemm_tc(CGemm g, Dft3 f, int *
       const uint64_t ah = sdesc(a + j * kHalfA), al = sdesc(a + (2 + j) * kHalfA);
       const int blk = KIND == 0 ? 1 - j : (KIND == 1 ? 2 * j : j);
       const uint64_t bh = sdesc(q + blk * kBlockB), bl = sdesc(q + kLoB + blk * kBlockB);
-      if (PREC == 1) mma<PREC>(dt, ah, bh, id, acc0);
-      mma<PREC>(dt, ah, bl, id, PREC == 1 ? 1u : acc0);
+      if (PREC != 2) mma<PREC>(dt, ah, bh, id, acc0);
+      mma<PREC>(dt, ah, bl, id, PREC != 2 ? 1u : acc0);
       mma<PREC>(dt, al, bh, id, 1u);
     }
-    if (PREC != 1) {
+    if (PREC == 2) {
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int blk = KIND == 0 ? 1 - j : (KIND == 1 ? 2 * j : j);
